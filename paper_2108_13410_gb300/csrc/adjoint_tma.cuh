@@ -52,7 +52,7 @@ __device__ __forceinline__ void adj_rotate_w(u64 (&p)[NR], u64 (&l)[NR], unsigne
     }
 }
 
-// Tangent form (records from dev_tan_triple): the inverse factor is cos th [[1, -t],
+// Tangent form (records from dev_tan): the inverse factor is cos th [[1, -t],
 // [t, 1]]; C = prod cos th is applied first (with the inverse Z layer, through the
 // conjugated scaled table, or alone for a group without Z), so when stage s reads its
 // terms psi and lambda both still carry prod cos th over the X qubits not yet

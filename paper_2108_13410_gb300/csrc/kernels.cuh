@@ -508,26 +508,54 @@ struct RecGeom {
 
 struct DevCouplings { double J, h, g, lambda; };
 
-__device__ inline void dev_unit_pair(bool f32, double t, double *ou, double *os) {
-    double sh = sin(0.5 * t);
-    double u = 2.0 * sh * sh, s = sin(t);
-    if (!f32) { *ou = u; *os = s; return; }
-    float u0 = (float)u, s0 = (float)s, bu = u0, bs = s0;
-    double c0 = 1.0 - (double)u0;
-    double be = fabs(c0 * c0 + (double)s0 * (double)s0 - 1.0), bd = 0.0;
-    float uu = u0;
-    for (int i = 0; i < 3; ++i) uu = nextafterf(uu, -4.0f);
-    for (int i = -3; i <= 3; ++i, uu = nextafterf(uu, 4.0f)) {
+// The float pair within +-3 ulps of (u, s) that minimises |(1 - u)^2 + s^2 - m2|, the first
+// of equal ones by distance from (u, s).  With e0 the deviation of the rounded pair (FP64),
+// the deviation of a neighbour is e0 + du (du - 2 (1 - u0)) + ds (ds + 2 s0) with du, ds the
+// (exact) float differences, evaluated in FP32 to ~1e-14: far below the ~1e-10 that the best
+// of the 49 pairs reaches, so FP64 runs once per entry instead of 49 times.  GB300 retires
+// about two FP64 FMAs per clock per SM and the search in FP64 was almost all of
+// k_build_records (100 us for the two factor groups of one 18-qubit step).
+__device__ inline void dev_nearest_modulus(double u, double s, double m2, double *ou, double *os) {
+    const float u0 = (float)u, s0 = (float)s;
+    const double c0 = 1.0 - (double)u0;
+    const float e0 = (float)(c0 * c0 + (double)s0 * (double)s0 - m2);
+    const float ru = (float)(u - (double)u0), rs = (float)(s - (double)s0);
+    const float a = -2.0f * (float)c0, b = 2.0f * s0;
+    float ds[7], es[7];
+    {
         float ss = s0;
-        for (int j = 0; j < 3; ++j) ss = nextafterf(ss, -4.0f);
-        for (int j = -3; j <= 3; ++j, ss = nextafterf(ss, 4.0f)) {
-            double c = 1.0 - (double)uu;
-            double e = fabs(c * c + (double)ss * (double)ss - 1.0);
-            double dd = fabs((double)uu - u) + fabs((double)ss - s);
-            if (e < be || (e == be && dd < bd)) { be = e; bd = dd; bu = uu; bs = ss; }
+        ds[3] = 0.f;
+#pragma unroll
+        for (int j = 2; j >= 0; --j) { ss = nextafterf(ss, -4.0f); ds[j] = ss - s0; }
+        ss = s0;
+#pragma unroll
+        for (int j = 4; j < 7; ++j) { ss = nextafterf(ss, 4.0f); ds[j] = ss - s0; }
+#pragma unroll
+        for (int j = 0; j < 7; ++j) es[j] = ds[j] * (ds[j] + b);
+    }
+    float be = fabsf(e0), bd = 0.f, bu = 0.f, bs = 0.f;
+    float uu = nextafterf(nextafterf(nextafterf(u0, -4.0f), -4.0f), -4.0f);
+    for (int i = 0; i < 7; ++i, uu = nextafterf(uu, 4.0f)) {
+        const float du = uu - u0;
+        const float eu = e0 + du * (du + a), dd = fabsf(du - ru);
+#pragma unroll
+        for (int j = 0; j < 7; ++j) {
+            const float e = fabsf(eu + es[j]), d = dd + fabsf(ds[j] - rs);
+            if (e < be || (e == be && d < bd)) { be = e; bd = d; bu = du; bs = ds[j]; }
         }
     }
-    *ou = bu; *os = bs;
+    *ou = (double)(u0 + bu); *os = (double)(s0 + bs);
+}
+
+__device__ inline void dev_unit_pair(bool f32, double t, double *ou, double *os) {
+    if (!f32) {
+        const double sh = sin(0.5 * t);
+        *ou = 2.0 * sh * sh; *os = sin(t);
+        return;
+    }
+    double sh, ch;
+    sincos(0.5 * t, &sh, &ch);
+    dev_nearest_modulus(2.0 * sh * sh, 2.0 * sh * ch, 1.0, ou, os);
 }
 
 // Careful pair of exp(i t) = (1 - u) + i s for per-step tables built inside a kernel:
@@ -605,12 +633,14 @@ __device__ inline void dev_op_angles(const RecGeom &G, const DevCouplings *__res
 // applied through the scaled Z table (dev_scaled_pair) or, for a factor group without
 // a Z layer, rounded once.  Used when |th| <= pi/4 and C >= 1/2 (the host checks;
 // otherwise the (u, s) form runs).  o = [t0, t1, C, 0].
-__device__ inline void dev_tan_triple(bool f32, double th0, double th1, int n0, int n1, double *o) {
-    double t0 = tan(th0), t1 = tan(th1);
-    if (f32) { t0 = (double)(float)t0; t1 = (double)(float)t1; }
-    o[0] = t0; o[1] = t1;
-    o[2] = pow(1.0 + t0 * t0, -0.5 * n0) * pow(1.0 + t1 * t1, -0.5 * n1);
-    o[3] = 0.0;
+__device__ inline void dev_tan(bool f32, double th, int n, double *t, double *f) {
+    double v = tan(th);
+    if (f32) v = (double)(float)v;
+    *t = v;
+    double x = 1.0 + v * v, p = 1.0;      // (1 + t^2)^n by squaring
+    for (; n; n >>= 1, x *= x)
+        if (n & 1) p *= x;
+    *f = p;
 }
 
 // C exp(i phi) as (u, s) with (1 - u) + i s, u = 1 - C cos phi, s = C sin phi; for
@@ -618,67 +648,63 @@ __device__ inline void dev_tan_triple(bool f32, double th0, double th1, int n0, 
 // |(1 - u)^2 + s^2 - C^2| (in double), so the modulus of every table entry is C to
 // ~1e-10 relative, as the unit pairs of dev_unit_pair are 1.
 __device__ inline void dev_scaled_pair(bool f32, double phi, double C, double *ou, double *os) {
-    const double sh = sin(0.5 * phi);
-    const double u = (1.0 - C) + C * 2.0 * sh * sh, s = C * sin(phi);
-    if (!f32) { *ou = u; *os = s; return; }
-    const double C2 = C * C;
-    float u0 = (float)u, s0 = (float)s, bu = u0, bs = s0;
-    double c0 = 1.0 - (double)u0;
-    double be = fabs(c0 * c0 + (double)s0 * (double)s0 - C2), bd = 0.0;
-    float uu = u0;
-    for (int i = 0; i < 3; ++i) uu = nextafterf(uu, -4.0f);
-    for (int i = -3; i <= 3; ++i, uu = nextafterf(uu, 4.0f)) {
-        float ss = s0;
-        for (int j = 0; j < 3; ++j) ss = nextafterf(ss, -4.0f);
-        for (int j = -3; j <= 3; ++j, ss = nextafterf(ss, 4.0f)) {
-            const double c = 1.0 - (double)uu;
-            const double e = fabs(c * c + (double)ss * (double)ss - C2);
-            const double dd = fabs((double)uu - u) + fabs((double)ss - s);
-            if (e < be || (e == be && dd < bd)) { be = e; bd = dd; bu = uu; bs = ss; }
-        }
+    if (!f32) {
+        const double sh = sin(0.5 * phi);
+        *ou = (1.0 - C) + C * 2.0 * sh * sh; *os = C * sin(phi);
+        return;
     }
-    *ou = bu; *os = bs;
+    double sh, ch;
+    sincos(0.5 * phi, &sh, &ch);
+    dev_nearest_modulus((1.0 - C) + C * 2.0 * sh * sh, C * 2.0 * sh * ch, C * C, ou, os);
 }
 
-// one thread per (op, batch, entry); entry 0 = X header, then Z table, then X table;
-// records of ops op0 .. op0 + n_ops - 1 are written from recs[0]
-__global__ void k_build_records(RecGeom G, const DevCouplings *__restrict__ cpl, const double *__restrict__ sv,
-                                int op0, int n_ops, double *__restrict__ recs) {
+// One record per blockIdx.x = (op - op0) * batch + b; its entries (0 = X header, then the Z
+// table, the X table, the Z table scaled by the tangent form's C) go to the threads of
+// blockIdx.y = 0, 1, ... in turn, and every block takes the group's angles and tangent
+// triple once into shared memory (the triple per entry was a third of the FP64 work).
+// Blocks of 64 threads: FP64 issue bounds the kernel, so a short call spreads over SMs.
+constexpr int REC_THREADS = 64;
+__global__ void __launch_bounds__(REC_THREADS) k_build_records(RecGeom G, const DevCouplings *__restrict__ cpl,
+                                                               const double *__restrict__ sv, int op0,
+                                                               double *__restrict__ recs) {
     const int nz = (G.nA + 1) * (G.nB + 1);
     const int nx = G.xlut_off > 0 ? (G.nXA + 1) * (G.nXB + 1) : 0;
     const int nt = G.tan_off > 0 ? nz : 0;
-    const long long per = 1 + nz + nx + nt;
-    const long long total = (long long)n_ops * G.batch * per;
-    for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < total;
-         id += (long long)gridDim.x * blockDim.x) {
-        const long long ob = id / per;
-        const int e = (int)(id - ob * per);
-        const int op = op0 + (int)(ob / G.batch), b = (int)(ob % G.batch);
-        double thx[2], zA, zB;
-        bool has_z;
-        dev_op_angles(G, cpl, b, sv, op, thx, &zA, &zB, &has_z);
-        double *r = recs + ob * G.rec_stride;
+    const int per = 1 + nz + nx + nt;
+    const long long ob = blockIdx.x;
+    const int op = op0 + (int)(ob / G.batch), b = (int)(ob % G.batch);
+    __shared__ double tri[2][2];        // per X class: t, (1 + t^2)^n
+    double thx[2], zA, zB;
+    bool has_z;
+    dev_op_angles(G, cpl, b, sv, op, thx, &zA, &zB, &has_z);
+    if (nt && threadIdx.x < 2)
+        dev_tan(G.f32, thx[threadIdx.x], threadIdx.x ? G.nX1 : G.nX0, &tri[threadIdx.x][0], &tri[threadIdx.x][1]);
+    __syncthreads();
+    const double C = nt ? 1.0 / sqrt(tri[0][1] * tri[1][1]) : 1.0;
+    double *r = recs + ob * G.rec_stride;
+    for (int e = blockIdx.y * REC_THREADS + threadIdx.x; e < per; e += gridDim.y * REC_THREADS) {
         if (e == 0) {
             dev_unit_pair(G.f32, thx[0], &r[0], &r[1]);
             dev_unit_pair(G.f32, thx[1], &r[2], &r[3]);
-            if (G.tan_off > 0) dev_tan_triple(G.f32, thx[0], thx[1], G.nX0, G.nX1, &r[G.tan_off]);
-        } else if (e <= nz) {
-            const int k = e - 1, a = k / (G.nB + 1), bb = k % (G.nB + 1);
-            double phi = has_z ? zA * (double)(G.nA - 2 * a) + zB * (double)(G.nB - 2 * bb) : 0.0;
-            dev_unit_pair(G.f32, phi, &r[4 + 2 * k], &r[5 + 2 * k]);
-        } else if (e <= nz + nx) {
-            const int k = e - 1 - nz, a = k / (G.nXB + 1), bb = k % (G.nXB + 1);
-            double phi = thx[1] * (double)(G.nXA - 2 * a) + thx[0] * (double)(G.nXB - 2 * bb);
-            dev_unit_pair(G.f32, phi, &r[G.xlut_off + 2 * k], &r[G.xlut_off + 2 * k + 1]);
-        } else {
-            // Z table scaled by the tangent form's C
-            const int k = e - 1 - nz - nx, a = k / (G.nB + 1), bb = k % (G.nB + 1);
-            double tc[4];
-            dev_tan_triple(G.f32, thx[0], thx[1], G.nX0, G.nX1, tc);
-            double phi = has_z ? zA * (double)(G.nA - 2 * a) + zB * (double)(G.nB - 2 * bb) : 0.0;
-            double *tl = r + G.tan_off + 4;
-            dev_scaled_pair(G.f32, phi, tc[2], &tl[2 * k], &tl[2 * k + 1]);
+            if (nt) {
+                double *o = r + G.tan_off;
+                o[0] = tri[0][0]; o[1] = tri[1][0]; o[2] = C; o[3] = 0.0;
+            }
+            continue;
         }
+        int k = e - 1;
+        const bool x_table = k >= nz && k < nz + nx;
+        const bool scaled = k >= nz + nx;
+        if (x_table) k -= nz;
+        else if (scaled) k -= nz + nx;
+        const int nb1 = (x_table ? G.nXB : G.nB) + 1;
+        const int a = k / nb1, bb = k % nb1;
+        double phi;
+        if (x_table) phi = thx[1] * (double)(G.nXA - 2 * a) + thx[0] * (double)(G.nXB - 2 * bb);
+        else phi = has_z ? zA * (double)(G.nA - 2 * a) + zB * (double)(G.nB - 2 * bb) : 0.0;
+        double *o = r + (x_table ? G.xlut_off : scaled ? G.tan_off + 4 : 4) + 2 * k;
+        if (scaled) dev_scaled_pair(G.f32, phi, C, &o[0], &o[1]);
+        else dev_unit_pair(G.f32, phi, &o[0], &o[1]);
     }
 }
 

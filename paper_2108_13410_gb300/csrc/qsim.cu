@@ -929,11 +929,15 @@ qs_status build_records(qs_sim *s, size_t op0, size_t n, double dt, int n_steps,
     G.tan_off = (s->lat.gauge_higgs && (s->dtype == QS_C64 || s->tan_active)) ? s->tan_off : 0;
     G.nX0 = s->nX0; G.nX1 = s->nX1;
     G.dt = dt;
-    long long entries = (long long)n * B * (1 + (G.tan_off ? 2 : 1) * (s->nA + 1) * (s->nB + 1) +
-                                            (G.xlut_off ? (s->nXA + 1) * (s->nXB + 1) : 0));
-    unsigned blocks = (unsigned)std::min<long long>((entries + 255) / 256, 152 * 16);
-    k_build_records<<<blocks, 256, 0, s->stream>>>(G, reinterpret_cast<const DevCouplings *>(s->d_in),
-                                                   s->d_in + 4 * s->in_ncpl, (int)op0, (int)n, s->d_rec);
+    const int entries = 1 + (G.tan_off ? 2 : 1) * (s->nA + 1) * (s->nB + 1) +
+                        (G.xlut_off ? (s->nXA + 1) * (s->nXB + 1) : 0);
+    // short calls: one entry per thread over many SMs; from about eight blocks per SM on a
+    // block takes its whole record, which shares the angles and the tangent triple
+    const long long slices = (entries + REC_THREADS - 1) / REC_THREADS;
+    const long long recs = (long long)n * B;
+    const unsigned gy = (unsigned)std::max<long long>(1, std::min<long long>(slices, 8ll * s->sm_count / recs));
+    k_build_records<<<dim3((unsigned)recs, gy), REC_THREADS, 0, s->stream>>>(
+        G, reinterpret_cast<const DevCouplings *>(s->d_in), s->d_in + 4 * s->in_ncpl, (int)op0, s->d_rec);
     CKL(s);
     s->launches++;
     return QS_OK;

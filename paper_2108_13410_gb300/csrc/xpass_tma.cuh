@@ -24,6 +24,7 @@
 #include <type_traits>
 
 #include "kernels.cuh"
+#include "packed.cuh"
 
 namespace qsim {
 
@@ -132,21 +133,6 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     return d;
 }
 
-typedef unsigned long long u64;
-
-__device__ __forceinline__ u64 pk(float x, float y) {
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-
-// packed FP32x2 FMA on register pairs
-__device__ __forceinline__ u64 fma2p(u64 a, u64 b, u64 c) {
-    u64 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
 __device__ __forceinline__ void rrotp(u64 &a, u64 &b, u64 nu, u64 ps, u64 ns) {
     const u64 ta = fma2p(nu, a, a);
     const u64 tb = fma2p(nu, b, b);
@@ -205,12 +191,6 @@ __device__ __forceinline__ void hadamard_regs2(float2 (&v)[NR], unsigned mask) {
     }
 }
 
-__device__ __forceinline__ float2 unpk(u64 w) {
-    float2 v;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(w));
-    return v;
-}
-
 // Real-frame rotations on packed register pairs; per class the constants
 // (-u, -u), (s, s), (-s, -s) are prepared once per operator record.
 struct RotConst { u64 nu[2], ps[2], ns[2]; };
@@ -227,7 +207,7 @@ __device__ __forceinline__ void rotate_w(u64 (&w)[NR], unsigned mask, const int 
     }
 }
 
-// Tangent form (dev_tan_triple): butterflies a' = a + t b, b' = b - t a on packed
+// Tangent form (dev_tan): butterflies a' = a + t b, b' = b - t a on packed
 // register pairs, constants (t, t) and (-t, -t) per class; the cos factors of the whole
 // X layer are applied once, as the record's scalar C.
 struct TanConst { u64 pt[2], nt[2]; };
@@ -301,13 +281,6 @@ __device__ __forceinline__ void hadamard_w(u64 (&w)[NR], unsigned mask) {
                 w[q] = fma2p(mone, b, a);
             }
     }
-}
-
-// v * i^k
-__device__ __forceinline__ float2 mul_ipow(float2 v, int k) {
-    float2 r = (k & 1) ? make_float2(-v.y, v.x) : v;
-    if (k & 2) { r.x = -r.x; r.y = -r.y; }
-    return r;
 }
 
 // MERGED: the pass applies X(G) of one factor group, the Z layer, then X(G) of the
