@@ -86,8 +86,12 @@ typedef enum {
     QS_OPT_PROFILE = 2,       /* 1: time every fused X-pass launch with CUDA events on
                                  the bound stream (read with qs_profile_read)        */
     QS_OPT_GRAPH = 3,         /* 1: qs_evolve replays its launches as a CUDA graph    */
-    QS_OPT_XPASS = 4,         /* X-pass kernel for complex64: 0 auto (TMA), 1 the
-                                 register-staged kernel, 2 the persistent TMA kernel */
+    QS_OPT_XPASS = 4,         /* X-pass kernel: 0 auto: calls of twelve or more factor
+                                 groups on small states (up to 2^19 amplitudes in all;
+                                 any number of states of up to 12 qubits) run in one
+                                 launch with the state on the chip, others as 2; 1 the
+                                 register-staged kernel, 2 the persistent TMA kernel
+                                 (complex64; complex128: the double-float passes)    */
     QS_OPT_TMA_BUFFERS = 5,   /* shared-memory tile buffers per CTA of the TMA kernel:
                                  2 (three CTAs per SM) or 3 (default; two CTAs per SM) */
     QS_OPT_ADJOINT = 6,       /* complex64 adjoint reverse pass: bit 0 set = register-
@@ -156,7 +160,8 @@ typedef enum {
 /* Create a simulator for an Lx x Ly lattice.  Periodic needs Lx, Ly >= 2; open
  * needs Lx, Ly >= 1.  batch >= 1 independent states share the lattice; each has
  * its own couplings.  Fails with QS_ERR_ARG if the qubit count exceeds 34.
- * Allocates only small device workspaces (term tables, partial sums). */
+ * Allocates only small device workspaces (term tables, partial sums; at the first
+ * call that runs on the chip, two mail boxes of at most 2^19 amplitudes each). */
 qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch,
                     qs_sim **out);
 void qs_destroy(qs_sim *sim);

@@ -26,6 +26,7 @@
 #include "adjoint_wl.cuh"
 #include "scan.cuh"
 #include "scan_mixed.cuh"
+#include "resident.h"
 
 using namespace qsim;
 
@@ -103,6 +104,12 @@ struct qs_sim {
     int tan_off = 0;                       // tangent triple in the operator record
     int nX0 = 0, nX1 = 0;                  // X qubits per class
     bool tan_active = false;               // this call's X passes use the tangent form
+    // small states: the whole run of factor groups in one launch (resident.cu)
+    ResParams res;
+    int res_known = 0;                     // 0 not looked at yet, 1 the state fits, -1 it does not
+    bool res_active = false;               // this call runs resident
+    void *d_res_mail = nullptr;            // its mail boxes (allocated at the first call that needs them)
+    bool res_mail_ready = false;           // cleared, and no launch on them has timed out since
     int adj_impl = 0;                      // adjoint reverse pass: 0 auto (TMA), 1 register kernel
     int adj_early = 1;                     // one buffer, tangent form: next load issued before the stores
     int sm_count = 0;
@@ -828,6 +835,7 @@ qs_status check_device_flag(qs_sim *s) {
     CK(s, cudaMemcpy(&flag, s->d_err, sizeof(int), cudaMemcpyDeviceToHost));
     if (flag) {
         cudaMemset(s->d_err, 0, sizeof(int));
+        s->res_mail_ready = false;
         FAIL(s, QS_ERR_TIMEOUT, "a bounded device wait gave up (flag %d)", flag);
     }
     return QS_OK;
@@ -914,21 +922,27 @@ qs_status upload_inputs(qs_sim *s, const qs_couplings *c, const double *sv, int 
     return QS_OK;
 }
 
+RecGeom record_geometry(const qs_sim *s, double dt, int n_steps, int order) {
+    RecGeom G;
+    memset(&G, 0, sizeof(G));
+    G.n_steps = n_steps; G.order = order; G.fsal = (order == 2); G.path = s->in_path ? 1 : 0;
+    G.batch = s->batch; G.rec_stride = s->rec_stride;
+    G.nA = s->nA; G.nB = s->nB; G.nXA = s->nXA; G.nXB = s->nXB;
+    G.xlut_off = s->lat.gauge_higgs ? 0 : s->xlut_off;
+    G.f32 = s->dtype == QS_C64;
+    G.nX0 = s->nX0; G.nX1 = s->nX1;
+    G.dt = dt;
+    return G;
+}
+
 qs_status build_records(qs_sim *s, size_t op0, size_t n, double dt, int n_steps, int order) {
     const int B = s->batch;
     qs_status st;
     if ((st = grow(s, &s->d_rec, &s->d_rec_cap, n * B * (size_t)s->rec_stride, false)) != QS_OK) return st;
-    RecGeom G;
-    G.n_steps = n_steps; G.order = order; G.fsal = (order == 2); G.path = s->in_path ? 1 : 0;
-    G.batch = B; G.rec_stride = s->rec_stride;
-    G.nA = s->nA; G.nB = s->nB; G.nXA = s->nXA; G.nXB = s->nXB;
-    G.xlut_off = s->lat.gauge_higgs ? 0 : s->xlut_off;
-    G.f32 = s->dtype == QS_C64;
+    RecGeom G = record_geometry(s, dt, n_steps, order);
     // tangent records only where the tangent form can run (gauge-Higgs; complex128 with
     // double-float passes)
     G.tan_off = (s->lat.gauge_higgs && (s->dtype == QS_C64 || s->tan_active)) ? s->tan_off : 0;
-    G.nX0 = s->nX0; G.nX1 = s->nX1;
-    G.dt = dt;
     const int entries = 1 + (G.tan_off ? 2 : 1) * (s->nA + 1) * (s->nB + 1) +
                         (G.xlut_off ? (s->nXA + 1) * (s->nXB + 1) : 0);
     // short calls: one entry per thread over many SMs; from about eight blocks per SM on a
@@ -939,6 +953,19 @@ qs_status build_records(qs_sim *s, size_t op0, size_t n, double dt, int n_steps,
     k_build_records<<<dim3((unsigned)recs, gy), REC_THREADS, 0, s->stream>>>(
         G, reinterpret_cast<const DevCouplings *>(s->d_in), s->d_in + 4 * s->in_ncpl, (int)op0, s->d_rec);
     CKL(s);
+    s->launches++;
+    return QS_OK;
+}
+
+// Records of a call's factor groups [op0, op0 + n) in the format of the kernels it runs on.
+qs_status build_call_records(qs_sim *s, size_t op0, size_t n, double dt, int n_steps, int order) {
+    if (!s->res_active) return build_records(s, op0, n, dt, n_steps, order);
+    qs_status st;
+    const ResParams &P = s->res;
+    const size_t bytes = n * s->batch * (size_t)P.rec_bytes;
+    if ((st = grow(s, &s->d_rec, &s->d_rec_cap, (bytes + 7) / 8, false)) != QS_OK) return st;
+    CK(s, resident_tables(P, record_geometry(s, dt, n_steps, order), reinterpret_cast<const DevCouplings *>(s->d_in),
+                          s->d_in + 4 * s->in_ncpl, (int)op0, (int)n, s->d_rec, s->sm_count, s->stream));
     s->launches++;
     return QS_OK;
 }
@@ -1056,6 +1083,94 @@ bool df_schedule(const qs_sim *s) {
            s->passes.size() >= 2 && (!s->lat.gauge_higgs || s->tan_active);
 }
 
+// Resident evolution: complex64, and complex128 in FP64 up to 12 qubits and in double-float
+// arithmetic from 13 on (where the tiled passes use it too).  States of one tile always: a
+// launch per pass takes twice as long at 12 qubits whatever the batch, and below 12 qubits
+// there are only per-factor kernels.  Otherwise as long as the latency of the passes is what
+// counts, 2^19 amplitudes in all; beyond, the tiled passes stream better.  Measured, resident
+// over passes per step: complex64 2^19 amplitudes 0.66 (19 qubits), 0.59 (4 x 17), 0.77 (64 x
+// 13), 2^20 1.12 (20 qubits), 1.15 (4 x 18), 1.64 (16 x 16); double-float 2^18 0.48 (18 qubits),
+// 0.72 (4 x 16), 2^19 0.69 (19 qubits), 0.75 (4 x 17) but 1.4 (64 x 13), 2^20 1.24 (4 x 18);
+// FP64 2^18 0.37 to 0.51 (64 x 12).
+constexpr size_t RES_MIN_GROUPS = 12;
+
+bool resident_size(const qs_sim *s) {
+    if (s->n < LT || (s->n == LT && s->dtype == QS_C64)) return true;
+    const long long amps = (long long)s->batch << s->n;
+    if (s->dtype == QS_C128 && s->n > LT && s->batch > 4) return amps <= 1ll << 18;
+    return amps <= 1ll << 19;
+}
+
+bool resident_fits(qs_sim *s) {
+    if (s->res_known == 0) {
+        s->res_known = -1;
+        ResParams &P = s->res;
+        memset(&P, 0, sizeof(P));
+        const int n = s->n;
+        if (!resident_size(s)) return false;
+        P.had = !s->lat.gauge_higgs;
+        P.nA = s->nA; P.nB = s->nB; P.nXA = s->nXA; P.nXB = s->nXB;
+        for (int q = 0; q < n; ++q) {
+            for (int p = 0; p < s->nA; ++p) if ((s->lat.plaquettes[p] >> q) & 1) P.colA[q] |= 1u << p;
+            for (int p = 0; p < s->nB; ++p) if ((s->lat.second[p] >> q) & 1) P.colB[q] |= 1u << p;
+            for (size_t v = 0; P.had && v < s->lat.stars.size(); ++v)
+                if ((s->lat.stars[v] >> q) & 1) P.xcolA[q] |= 1u << v;
+            P.xcolB[q] = 1u << q;
+            if (s->lat.x_class[q]) P.cls |= 1u << q;
+        }
+        const int arith = s->dtype == QS_C64 ? RES_F32 : n <= LT ? RES_F64 : RES_DF;
+        if (resident_plan(P, arith, n, s->batch, s->sm_count)) s->res_known = 1;
+    }
+    return s->res_known == 1;
+}
+
+qs_status resident_mail(qs_sim *s) {
+    const size_t bytes = resident_mail_bytes(s->res);
+    if (!bytes || s->res_mail_ready) return QS_OK;
+    if (!s->d_res_mail && cudaMalloc(&s->d_res_mail, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        s->d_res_mail = nullptr;
+        FAIL(s, QS_ERR_OOM, "mail boxes of %zu bytes", bytes);
+    }
+    CK(s, resident_mail_clear(s->res, s->d_res_mail, s->stream));
+    s->res_mail_ready = true;
+    return QS_OK;
+}
+
+// A call runs resident by default (QS_OPT_XPASS auto, shared passes on, the default pass
+// plan, no per-pass profiling) from RES_MIN_GROUPS factor groups on, and with as many
+// between renormalisations: shorter runs keep one launch per pass, whose number
+// qs_launch_count reports to callers.
+bool resident_call(qs_sim *s, size_t nops, int steps_per_renorm_unit) {
+    if (s->method != 0 || s->xpass_impl != 0 || !s->xmerge || s->profile || s->passes.size() > 2) return false;
+    if (s->dtype == QS_C128 && s->n > LT && !s->c128_df) return false;
+    if (nops < RES_MIN_GROUPS) return false;
+    if (s->renorm_every > 0 && (size_t)s->renorm_every * (size_t)std::max(1, steps_per_renorm_unit) < RES_MIN_GROUPS)
+        return false;
+    return resident_fits(s);
+}
+
+template <typename R>
+qs_status launch_ops_resident(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm_unit, size_t j0, size_t j1) {
+    qs_status st;
+    const int B = s->batch;
+    const size_t nops = ops.size() / B;
+    const size_t unit = (size_t)s->renorm_every * (size_t)std::max(0, steps_per_renorm_unit);
+    for (size_t k = j0; k < j1;) {
+        const size_t k1 = unit ? std::min(j1, (k / unit + 1) * unit) : j1;
+        ResParams P = s->res;
+        P.nops = (int)(k1 - k);
+        P.last_z = ops[(k1 - 1) * B].has_z ? 1 : 0;
+        CK(s, resident_launch(P, s->state[0], (char *)s->d_rec + (k - j0) * B * (size_t)P.rec_bytes, s->d_res_mail, s->d_err,
+                              s->stream));
+        s->launches++;
+        k = k1;
+        if (unit && (k % unit == 0 || k == nops))
+            if ((st = renormalise<R>(s)) != QS_OK) return st;
+    }
+    return QS_OK;
+}
+
 template <typename R>
 qs_status launch_ops(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm_unit, size_t j0 = 0,
                      size_t j1 = (size_t)-1) {
@@ -1063,6 +1178,7 @@ qs_status launch_ops(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm
     const int B = s->batch;
     const size_t nops = ops.size() / B;
     if (j1 > nops) j1 = nops;
+    if (s->res_active) return launch_ops_resident<R>(s, ops, steps_per_renorm_unit, j0, j1);
     if (merged_schedule<R>(s)) return launch_ops_merged<R>(s, ops, steps_per_renorm_unit, j0, j1);
     if (df_schedule<R>(s) && !s->df_active) {
         // split into the blocked double-float layout, run the passes, join back
@@ -1096,28 +1212,31 @@ qs_status run_ops(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm_un
     // bounded growth before C is applied, and the scaled Z table u = 1 - C cos phi stays
     // away from 1, where rounding u would cost relative precision in C
     s->tan_active = false;
+    s->res_active = resident_call(s, nops, steps_per_renorm_unit);
     const bool tma_path = sizeof(R) == 4 ? s->tmaps_ok : (s->c128_df && s->tmaps_df_ok);
-    if (s->method == 0 && s->lat.gauge_higgs && tma_path && s->xpass_impl != 1) {
+    if (s->method == 0 && s->lat.gauge_higgs && (tma_path || s->res_active) && s->xpass_impl != 1) {
         bool ok = true;
         for (const Op &o : ops) {
             const double t0 = std::tan(o.thx[0]), t1 = std::tan(o.thx[1]);
             ok = ok && std::fabs(o.thx[0]) <= 0.25 * M_PI && std::fabs(o.thx[1]) <= 0.25 * M_PI &&
                  s->nX0 * std::log1p(t0 * t0) + s->nX1 * std::log1p(t1 * t1) <= 2.0 * std::log(2.0);
         }
-        s->tan_active = ok;
+        s->tan_active = ok && tma_path;
+        s->res_active = s->res_active && ok;
     }
     if (s->method == 0) {
+        if (s->res_active && (st = resident_mail(s)) != QS_OK) return st;
         if ((st = upload_inputs(s, c, sv, n_steps, path)) != QS_OK) return st;
         if (nops > REC_CHUNK) {
             // long schedules: records of REC_CHUNK ops at a time, direct launches
             for (size_t j0 = 0; j0 < nops; j0 += REC_CHUNK) {
                 const size_t j1 = std::min(nops, j0 + REC_CHUNK);
-                if ((st = build_records(s, j0, j1 - j0, dt, n_steps, order)) != QS_OK) return st;
+                if ((st = build_call_records(s, j0, j1 - j0, dt, n_steps, order)) != QS_OK) return st;
                 if ((st = launch_ops<R>(s, ops, steps_per_renorm_unit, j0, j1)) != QS_OK) return st;
             }
             return QS_OK;
         }
-        if ((st = build_records(s, 0, nops, dt, n_steps, order)) != QS_OK) return st;
+        if ((st = build_call_records(s, 0, nops, dt, n_steps, order)) != QS_OK) return st;
     }
     if (!s->use_graph || s->profile) return launch_ops<R>(s, ops, steps_per_renorm_unit);
     // Replay the launch sequence as a CUDA graph, captured once per configuration on a
@@ -1126,7 +1245,7 @@ qs_status run_ops(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm_un
                                (long long)(uintptr_t)s->d_rec, s->renorm_every,
                                s->xpass_impl * 16 + s->nbuf + 256 * s->tma_store + 1024 * s->xmerge +
                                    4096 * (int)s->tan_active + 8192 * s->pdl + 16384 * s->nbuf_shared +
-                                   65536 * s->shared_kernel + 131072 * s->c128_df,
+                                   65536 * s->shared_kernel + 131072 * s->c128_df + 262144 * (int)s->res_active,
                                s->method, (long long)s->dtype};
     if (!s->graph_exec || memcmp(key, s->graph_key, sizeof(key)) != 0) {
         if (s->graph_exec) { cudaGraphExecDestroy(s->graph_exec); s->graph_exec = nullptr; }
@@ -1521,6 +1640,7 @@ void qs_destroy(qs_sim *s) {
     cudaFree(s->d_partials);
     cudaFree(s->d_res);
     cudaFree(s->d_err);
+    cudaFree(s->d_res_mail);
     cudaFree(s->d_adj_part);
     cudaFree(s->d_grad);
     cudaFree(s->d_hrec);
@@ -2135,6 +2255,8 @@ qs_status qs_autotune(qs_sim *s, int n_steps, int *best_xpass, int *best_buffers
         FAIL(s, QS_ERR_ARG, "null output");
     struct Cand { int xpass, nbuf, store, nsh, skern; };
     std::vector<Cand> cands;
+    if (s->passes.size() <= 2 && resident_fits(s))      // the default: resident, shared passes by form
+        cands.push_back({0, 3, 1, 0, 1});
     if (s->dtype == QS_C64 && s->tmaps_ok) {
         for (int nb = 2; nb <= 3; ++nb)
             for (int so = 0; so <= 1; ++so)
