@@ -399,93 +399,8 @@ __device__ __forceinline__ void block_store(double (&acc)[NVAL], double *out) {
     }
 }
 
-// values: [norm, sum_i p_i (nA - 2 oddA(i)), sum_i p_i (nB - 2 oddB(i)), <Z_zmask>],
-// p_i = |psi_i|^2.  Products are summed in the state's precision over runs of
-// RED_RUN amplitudes (exact enough: 8 terms of one sign-pattern), and the runs are
-// accumulated in FP64.
+// products summed in the state's precision before an accumulator takes them
 constexpr int RED_RUN = 8;
-
-template <typename R>
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_diag(
-    const typename C2<R>::T *__restrict__ psi, int n, long long state_stride,
-    const uint32_t *__restrict__ colA, const uint32_t *__restrict__ colB, int nA, int nB,
-    unsigned long long zmask, double *__restrict__ partials) {
-    __shared__ uint2 tab[MAXBYTES * 256];
-    psi += (long long)blockIdx.y * state_stride;
-    build_parity_tables(tab, colA, colB, n);
-    __syncthreads();
-    const int nbytes = (n + 7) / 8;
-    const long long dim = 1ll << n;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; i0 < dim; i0 += stride * RED_RUN) {
-        R f[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int u = 0; u < RED_RUN; ++u) {
-            long long i = i0 + u * stride;
-            if (i < dim) {
-                auto a = psi[i];
-                R p = a.x * a.x + a.y * a.y;
-                uint2 par = parity_of(tab, i, nbytes);
-                f[0] += p;
-                f[1] += p * (R)(nA - 2 * __popc(par.x));
-                f[2] += p * (R)(nB - 2 * __popc(par.y));
-                f[3] += (__popcll((unsigned long long)i & zmask) & 1) ? -p : p;
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[v] += (double)f[v];
-    }
-    block_store<4>(acc, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
-}
-
-// sum_i conj(a_i) b_{i ^ mask} (re, im); with a == b this is <X_mask>
-template <typename R>
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_xmask(
-    const typename C2<R>::T *__restrict__ a, const typename C2<R>::T *__restrict__ b, int n,
-    long long state_stride, unsigned long long mask, double *__restrict__ partials) {
-    a += (long long)blockIdx.y * state_stride;
-    b += (long long)blockIdx.y * state_stride;
-    const long long dim = 1ll << n;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    double acc[2] = {0.0, 0.0};
-    for (long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; i0 < dim; i0 += stride * RED_RUN) {
-        R f0 = 0, f1 = 0;
-#pragma unroll
-        for (int u = 0; u < RED_RUN; ++u) {
-            long long i = i0 + u * stride;
-            if (i < dim) {
-                auto x = a[i];
-                auto y = b[i ^ (long long)mask];
-                f0 += x.x * y.x + x.y * y.y;
-                f1 += x.x * y.y - x.y * y.x;
-            }
-        }
-        acc[0] += (double)f0;
-        acc[1] += (double)f1;
-    }
-    block_store<2>(acc, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
-}
-
-// res[b * RED_NV + v] = sum over the nblk partials of batch b (fixed order)
-__global__ void k_finish(const double *__restrict__ partials, int nblk, int nval,
-                         double *__restrict__ res) {
-    __shared__ double sh[RED_THREADS];
-    const int b = blockIdx.x;
-    for (int v = 0; v < nval; ++v) {
-        double s = 0.0;
-        for (int k = threadIdx.x; k < nblk; k += blockDim.x)
-            s += partials[((long long)b * nblk + k) * RED_NV + v];
-        sh[threadIdx.x] = s;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) res[b * RED_NV + v] = sh[0];
-        __syncthreads();
-    }
-}
 
 }  // namespace qsim
 
@@ -538,43 +453,6 @@ __global__ void __launch_bounds__(REC_THREADS) k_build_records(RecGeom G, const 
         double *o = r + (x_table ? G.xlut_off : scaled ? G.tan_off + 4 : 4) + 2 * k;
         if (scaled) dev_scaled_pair(G.f32, phi, C, &o[0], &o[1]);
         else dev_unit_pair(G.f32, phi, &o[0], &o[1]);
-    }
-}
-
-}  // namespace qsim
-
-namespace qsim {
-
-// Density of states of Z~ = -sum_l sigma^z_l (Sec. V): P(k) = sum over amplitudes with k
-// links in sigma^z = -1 of |psi_i|^2 (Z~ = 2k - n_links).  Per-block bins in shared
-// memory (FP64 atomics), then per-block partials; partials[(b * gridDim.x + blk) * nbins + k].
-template <typename R>
-__global__ void __launch_bounds__(RED_THREADS) k_dos(const typename C2<R>::T *__restrict__ psi, int n,
-                                                     long long state_stride, unsigned long long linkmask, int nbins,
-                                                     double *__restrict__ partials) {
-    __shared__ double bins[64];
-    for (int k = threadIdx.x; k < nbins; k += blockDim.x) bins[k] = 0.0;
-    __syncthreads();
-    psi += (long long)blockIdx.y * state_stride;
-    const long long dim = 1ll << n;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < dim;
-         i += (long long)gridDim.x * blockDim.x) {
-        auto a = psi[i];
-        double p = (double)a.x * (double)a.x + (double)a.y * (double)a.y;
-        atomicAdd(&bins[__popcll((unsigned long long)i & linkmask)], p);
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < nbins; k += blockDim.x)
-        partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * nbins + k] = bins[k];
-}
-
-// out[b * nval + v] = sum over nblk partials (layout [b][blk][v]), fixed order
-__global__ void k_finish_wide(const double *__restrict__ partials, int nblk, int nval, double *__restrict__ out) {
-    const int b = blockIdx.x;
-    for (int v = threadIdx.x; v < nval; v += blockDim.x) {
-        double s = 0.0;
-        for (int k = 0; k < nblk; ++k) s += partials[((long long)b * nblk + k) * nval + v];
-        out[(long long)b * nval + v] = s;
     }
 }
 

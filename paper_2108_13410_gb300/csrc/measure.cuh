@@ -1,0 +1,527 @@
+// measure.cuh -- reductions over a state: norm, diagonal sums, X strings, overlaps, the energy
+// terms and the density of states (sm_103a).
+//
+// All of them read the state and are bound by that where the arithmetic allows: GB300 retires
+// about two FP64 operations per clock and SM, so complex64 sums run in FP32 (products over
+// 16 amplitudes, then an error-free two-float accumulator per thread, converted to FP64 once
+// per block), the parity words of an amplitude are a tile word, a thread word and a register
+// word (no table look-up per amplitude), and of an X string only one amplitude of every pair
+// is visited.  Blocks write partial sums; k_finish adds them in a fixed order.
+// A tile is 4096 consecutive amplitudes (registers bits 8..11, threads bits 0..7) or, for the
+// X terms of the energy, one tile of an X pass (kernels.cuh).
+#pragma once
+#include "kernels.cuh"
+
+namespace qsim {
+
+// Per-thread accumulator: FP64, or for complex64 an unevaluated sum of two floats (Knuth's
+// two-sum keeps every rounding error, so it is as exact as FP64 partial sums of floats).
+template <typename R> struct Acc;
+template <> struct Acc<double> {
+    double h = 0.0;
+    __device__ __forceinline__ void add(double x) { h += x; }
+    __device__ __forceinline__ double value() const { return h; }
+};
+template <> struct Acc<float> {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
+        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
+        h = s;
+    }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
+// n - 2 k without a conversion instruction (quarter rate); k < 2^22.  FP64 sums take it from a
+// table in shared memory: the FP64 pipe is what bounds them.
+__device__ __forceinline__ float weight(const float *, float n, int k) {
+    return fmaf(-2.0f, __uint_as_float(0x4b000000u | (unsigned)k) - 8388608.0f, n);
+}
+__device__ __forceinline__ double weight(const double *tab, double, int k) { return tab[k]; }
+
+// tables of nA - 2 k and nB - 2 k (complex128)
+template <typename R>
+__device__ __forceinline__ void load_weights(R (*w)[33], int nA, int nB) {
+    if (sizeof(R) == 8)
+        for (int k = threadIdx.x; k < 66; k += blockDim.x) w[k / 33][k % 33] = (R)((k < 33 ? nA : nB) - 2 * (k % 33));
+}
+__device__ __forceinline__ float flip_sign(float x, unsigned odd) {
+    return __uint_as_float(__float_as_uint(x) ^ (odd << 31));
+}
+__device__ __forceinline__ double flip_sign(double x, unsigned odd) {
+    return __longlong_as_double(__double_as_longlong(x) ^ ((long long)odd << 63));
+}
+
+// Parity words of 4096-amplitude tiles: tile word from byte tables over bits 12.., thread word
+// over bits 0..7, register columns over bits 8..11.
+struct TileParity {
+    uint32_t ta, tb;          // thread
+    uint32_t ra[RB], rb[RB];  // register bits
+};
+
+__device__ __forceinline__ void load_tile_parity(TileParity &q, uint2 *tab, const uint32_t *colA, const uint32_t *colB,
+                                                 int n) {
+    const int t = threadIdx.x;
+    for (int e = t; e < 3 * 256; e += blockDim.x) {
+        uint32_t a = 0, b = 0;
+        for (int j = 0; j < 8; ++j) {
+            const int bit = LT + 8 * (e >> 8) + j;
+            if (bit < n && ((e >> j) & 1)) { a ^= colA[bit]; b ^= colB[bit]; }
+        }
+        tab[e] = make_uint2(a, b);
+    }
+    q.ta = q.tb = 0;
+#pragma unroll
+    for (int j = 0; j < TB; ++j)
+        if ((t >> j) & 1) { q.ta ^= colA[j]; q.tb ^= colB[j]; }
+#pragma unroll
+    for (int k = 0; k < RB; ++k) { q.ra[k] = colA[TB + k]; q.rb[k] = colB[TB + k]; }
+}
+
+__device__ __forceinline__ void tile_word(const uint2 *tab, long long tile, uint32_t &a, uint32_t &b) {
+    const uint2 x = tab[tile & 255], y = tab[256 + ((tile >> 8) & 255)], z = tab[512 + ((tile >> 16) & 255)];
+    a = x.x ^ y.x ^ z.x;
+    b = x.y ^ y.y ^ z.y;
+}
+
+// |psi|^2 sums of one amplitude set: f[0] norm, and if SUMS f[1], f[2] weighted by nA - 2 oddA,
+// nB - 2 oddB
+template <typename R, bool SUMS>
+__device__ __forceinline__ void diag_terms(R p, uint32_t a, uint32_t b, const R (*w)[33], R nA, R nB, R (&f)[4]) {
+    f[0] += p;
+    if (SUMS) {
+        f[1] = fma(p, weight(w[0], nA, __popc(a)), f[1]);
+        f[2] = fma(p, weight(w[1], nB, __popc(b)), f[2]);
+    }
+}
+
+// partial sums [norm, sum_i p_i (nA - 2 oddA(i)), sum_i p_i (nB - 2 oddB(i)), <Z_zmask>], p = |psi|^2
+// (the middle two only if SUMS, the last only if Z).  27 qubits in complex64: 0.15 ms, 0.21 with
+// the sums (0.16 at the measured copy rate); 0.66 ms with four table look-ups per amplitude and
+// an FP64 add per eight amplitudes and value.  24 qubits in complex128 (FP64-bound): 0.10 ms
+// for the norm, 0.31 before.
+template <typename R, bool SUMS, bool Z>
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_diag(const typename C2<R>::T *__restrict__ psi, int n,
+                                                            long long state_stride, const uint32_t *__restrict__ colA,
+                                                            const uint32_t *__restrict__ colB, int nA, int nB,
+                                                            unsigned long long zmask, double *__restrict__ partials) {
+    using V = typename C2<R>::T;
+    __shared__ uint2 tab[3 * 256];
+    __shared__ R wt[2][33];
+    TileParity q;
+    if (SUMS) {
+        load_tile_parity(q, tab, colA, colB, n);
+        load_weights<R>(wt, nA, nB);
+    }
+    __syncthreads();
+    psi += (long long)blockIdx.y * state_stride;
+    const int t = threadIdx.x;
+    const long long dim = 1ll << n, ntiles = n > LT ? dim >> LT : 1;
+    const unsigned zt = __popc(t & (unsigned)zmask & 255u);
+    Acc<R> acc[4];
+    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const V *p0 = psi + (tile << LT) + t;
+        V v[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            v[r] = n >= LT || (r << TB) + t < dim ? p0[r << TB] : mk<R>((R)0, (R)0);
+        uint32_t ta = 0, tb = 0;
+        if (SUMS) { tile_word(tab, tile, ta, tb); ta ^= q.ta; tb ^= q.tb; }
+        const unsigned zz = zt + __popcll(((unsigned long long)tile << LT) & zmask);
+        R f[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const R p = fma(v[r].y, v[r].y, v[r].x * v[r].x);
+            uint32_t a = ta, b = tb;
+            if (SUMS) {
+#pragma unroll
+                for (int k = 0; k < RB; ++k)
+                    if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
+            }
+            diag_terms<R, SUMS>(p, a, b, wt, (R)nA, (R)nB, f);
+            if (Z) f[3] += flip_sign(p, (zz + __popc((unsigned)(zmask >> TB) & (unsigned)r)) & 1u);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k == 0 || (SUMS && k < 3) || (Z && k == 3)) acc[k].add(f[k]);
+    }
+    double out[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[k] = acc[k].value();
+    block_store<4>(out, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
+}
+
+// <X_mask> (mask != 0): twice the real part over the pairs, each visited once at its member
+// with the mask's top bit clear: 0.15 ms at 27 qubits in complex64, 0.49 when every amplitude
+// fetched its partner; 0.06 and 0.21 at 24 qubits in complex128.
+template <typename R>
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_xpair(const typename C2<R>::T *__restrict__ psi, int n,
+                                                             long long state_stride, unsigned long long mask, int top,
+                                                             double *__restrict__ partials) {
+    using V = typename C2<R>::T;
+    psi += (long long)blockIdx.y * state_stride;
+    const long long pairs = 1ll << (n - 1), low = (1ll << top) - 1;
+    const long long stride = (long long)gridDim.x * RED_THREADS;
+    Acc<R> acc;
+    for (long long j0 = blockIdx.x * (long long)RED_THREADS + threadIdx.x; j0 < pairs; j0 += stride * RED_RUN) {
+        V x[RED_RUN], y[RED_RUN];
+#pragma unroll
+        for (int u = 0; u < RED_RUN; ++u) {
+            const long long j = j0 + u * stride;
+            const long long i = ((j & ~low) << 1) | (j & low);
+            x[u] = j < pairs ? psi[i] : mk<R>((R)0, (R)0);
+            y[u] = j < pairs ? psi[i ^ (long long)mask] : mk<R>((R)0, (R)0);
+        }
+        R f = 0;
+#pragma unroll
+        for (int u = 0; u < RED_RUN; ++u) f = fma(x[u].y, y[u].y, fma(x[u].x, y[u].x, f));
+        acc.add(f);
+    }
+    double out[2] = {2.0 * acc.value(), 0.0};
+    block_store<2>(out, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
+}
+
+// sum_i conj(a_i) b_i (re, im)
+template <typename R>
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_dot(const typename C2<R>::T *__restrict__ a,
+                                                           const typename C2<R>::T *__restrict__ b, int n,
+                                                           long long state_stride, double *__restrict__ partials) {
+    using V = typename C2<R>::T;
+    a += (long long)blockIdx.y * state_stride;
+    b += (long long)blockIdx.y * state_stride;
+    const long long dim = 1ll << n;
+    const long long stride = (long long)gridDim.x * RED_THREADS;
+    Acc<R> re, im;
+    for (long long i0 = blockIdx.x * (long long)RED_THREADS + threadIdx.x; i0 < dim; i0 += stride * RED_RUN) {
+        V x[RED_RUN], y[RED_RUN];
+#pragma unroll
+        for (int u = 0; u < RED_RUN; ++u) {
+            const long long i = i0 + u * stride;
+            x[u] = i < dim ? a[i] : mk<R>((R)0, (R)0);
+            y[u] = i < dim ? b[i] : mk<R>((R)0, (R)0);
+        }
+        R f0 = 0, f1 = 0;
+#pragma unroll
+        for (int u = 0; u < RED_RUN; ++u) {
+            f0 = fma(x[u].y, y[u].y, fma(x[u].x, y[u].x, f0));
+            f1 = fma(-x[u].y, y[u].x, fma(x[u].x, y[u].y, f1));
+        }
+        re.add(f0);
+        im.add(f1);
+    }
+    double out[2] = {re.value(), im.value()};
+    block_store<2>(out, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
+}
+
+// ---------------------------------------------------------------------------
+// Every term of <H> in one launch: partials [norm, sum Z_A, sum Z_B, sum X of class 0, of class
+// 1, 0, 0, 0].  Blocks take roles by blockIdx.x: pass p's tiles (pairs of the pass's qubits in
+// registers, through shared memory in the three stage layouts; the first pass also the
+// diagonal sums), then the X strings that no tile holds (stars of the unitary gauge; below 12
+// qubits all X terms, and the diagonal ones in a role of their own).  One read per pass plus
+// half a read per string.  27 qubits in complex64: 0.59 ms (three reads, 0.48 at the copy rate),
+// 1.5 with a diagonal pass of its own; 24 qubits with twelve stars in complex128: 1.6 ms (41 FP64
+// operations per amplitude), 4.2 with a reduction per star; 18 qubits with nine stars 25 us in
+// two launches, 150 in 24.
+// ---------------------------------------------------------------------------
+constexpr int EN_NV = 8;
+constexpr int EN_MASKS = 64;
+
+struct EnergyParams {
+    int n, np, gp, gm;             // qubits, passes, blocks per pass, blocks of the strings
+    int nA, nB, nmasks;
+    int c[4], next[4], k[4];       // passes: chunk bits, first new qubit, new qubits (first pass 12, 12, 0)
+    unsigned long long cls;        // bit q: qubit q is of class 1
+    unsigned long long mask[EN_MASKS];
+    unsigned long long mask_cls;   // bit j: string j is of class 1
+};
+
+template <typename R>
+__global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typename C2<R>::T *__restrict__ psi,
+                                                                    long long state_stride,
+                                                                    const uint32_t *__restrict__ colA,
+                                                                    const uint32_t *__restrict__ colB,
+                                                                    const __grid_constant__ EnergyParams P,
+                                                                    double *__restrict__ partials) {
+    using V = typename C2<R>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint2 tab[3 * 256];
+    __shared__ double sh[NT / 32][EN_NV];
+    __shared__ R wt[2][33];
+    V *tile_s = reinterpret_cast<V *>(smem_raw);
+    const int t = threadIdx.x;
+    const int roles = P.np * P.gp;
+    const int role = (int)blockIdx.x < roles ? (int)blockIdx.x / P.gp : P.np;
+    psi += (long long)blockIdx.y * state_stride;
+    const long long dim = 1ll << P.n, ntiles = P.n > LT ? dim >> LT : 1;
+    const bool diag = role == 0 || (P.np == 0 && (int)blockIdx.x < P.gm);
+    TileParity q;
+    if (diag) {
+        load_tile_parity(q, tab, colA, colB, P.n);
+        load_weights<R>(wt, P.nA, P.nB);
+    }
+    __syncthreads();
+    Acc<R> acc[5];
+    if (role < P.np) {
+        const int c = P.c[role], next = P.next[role];
+        auto g = [&](int j) { return j < c ? j : next + (j - c); };   // global bit of tile bit j
+        const unsigned rot = role == 0 ? (1u << LT) - 1 : ((1u << LT) - 1) & ~((1u << c) - 1);
+        unsigned cls = 0;
+        for (int j = 0; j < LT; ++j) cls |= (unsigned)((P.cls >> g(j)) & 1) << j;
+        const int mid = next - c, hi = next + P.k[role];
+        long long toff = 0, rs[RB];
+#pragma unroll
+        for (int j = 0; j < TB; ++j)
+            if ((t >> j) & 1) toff |= 1ll << g(j);
+#pragma unroll
+        for (int k = 0; k < RB; ++k) rs[k] = 1ll << g(TB + k);
+        auto load = [&](V (&v)[NR], long long tau) {
+            const V *p = psi + (((tau & ((1ll << mid) - 1)) << c) | ((tau >> mid) << hi)) + toff;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                long long off = 0;
+#pragma unroll
+                for (int k = 0; k < RB; ++k)
+                    if ((r >> k) & 1) off += rs[k];
+                v[r] = p[off];
+            }
+        };
+        auto pairs = [&](const V (&v)[NR], unsigned mask, unsigned cl, R &g0, R &g1) {
+#pragma unroll
+            for (int k = 0; k < RB; ++k) {
+                if (!((mask >> k) & 1u)) continue;
+                R s = 0;
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    if (!((r >> k) & 1)) s = fma(v[r].y, v[r | (1 << k)].y, fma(v[r].x, v[r | (1 << k)].x, s));
+                if ((cl >> k) & 1u) g1 += s; else g0 += s;
+            }
+        };
+        const int tlo = t & 15, thi = t >> 4;
+        V v[NR], u[NR];
+        const int b0 = (int)blockIdx.x - role * P.gp;
+        if (sizeof(R) == 4 && b0 < ntiles) load(u, b0);
+        for (long long tau = b0; tau < ntiles; tau += P.gp) {
+            if (sizeof(R) == 4) {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) v[r] = u[r];
+            } else {
+                load(v, tau);
+            }
+            R g0 = 0, g1 = 0;
+            if (role == 0) {
+                uint32_t ta, tb;
+                tile_word(tab, tau, ta, tb);
+                ta ^= q.ta; tb ^= q.tb;
+                R f[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    uint32_t a = ta, b = tb;
+#pragma unroll
+                    for (int k = 0; k < RB; ++k)
+                        if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
+                    diag_terms<R, true>(fma(v[r].y, v[r].y, v[r].x * v[r].x), a, b, wt, (R)P.nA, (R)P.nB, f);
+                }
+                acc[0].add(f[0]); acc[1].add(f[1]); acc[2].add(f[2]);
+            }
+            pairs(v, rot >> 8, cls >> 8, g0, g1);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) tile_s[swz(t | (r << TB))] = v[r];
+            __syncthreads();
+            // complex64: the next tile is on its way during the other two stages
+            if (sizeof(R) == 4 && tau + P.gp < ntiles) load(u, tau + P.gp);
+            if (rot & 15u) {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) v[r] = tile_s[swz(r | (t << RB))];
+                pairs(v, rot, cls, g0, g1);
+            }
+            if (rot & 0xf0u) {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) v[r] = tile_s[swz(tlo | (r << 4) | (thi << 8))];
+                pairs(v, rot >> 4, cls >> 4, g0, g1);
+            }
+            acc[3].add((R)2 * g0);
+            acc[4].add((R)2 * g1);
+            __syncthreads();
+        }
+    } else {
+        const int b0 = (int)blockIdx.x - roles;
+        for (long long tau = b0; tau < ntiles; tau += P.gm) {
+            V v[NR];
+            const long long i0 = (tau << LT) + t;
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+                v[r] = i0 + (r << TB) < dim ? psi[i0 + (r << TB)] : mk<R>((R)0, (R)0);
+            if (diag) {
+                uint32_t ta, tb;
+                tile_word(tab, tau, ta, tb);
+                ta ^= q.ta; tb ^= q.tb;
+                R f[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    uint32_t a = ta, b = tb;
+#pragma unroll
+                    for (int k = 0; k < RB; ++k)
+                        if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
+                    diag_terms<R, true>(fma(v[r].y, v[r].y, v[r].x * v[r].x), a, b, wt, (R)P.nA, (R)P.nB, f);
+                }
+                acc[0].add(f[0]); acc[1].add(f[1]); acc[2].add(f[2]);
+            }
+            for (int j = 0; j < P.nmasks; ++j) {
+                const long long m = (long long)P.mask[j];
+                const long long top = 1ll << (63 - __clzll(m));
+                R s = 0;
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    const long long i = i0 + (r << TB);
+                    if (i < dim && !(i & top)) {
+                        const V y = psi[i ^ m];
+                        s = fma(v[r].y, y.y, fma(v[r].x, y.x, s));
+                    }
+                }
+                if ((P.mask_cls >> j) & 1) acc[4].add((R)2 * s); else acc[3].add((R)2 * s);
+            }
+        }
+    }
+    const int w = t >> 5;
+#pragma unroll
+    for (int k = 0; k < EN_NV; ++k) {
+        const double x = k < 5 ? warp_sum(acc[k].value()) : 0.0;
+        if ((t & 31) == 0) sh[w][k] = x;
+    }
+    __syncthreads();
+    if (t < EN_NV) {
+        double s = 0.0;
+        for (int k = 0; k < NT / 32; ++k) s += sh[k][t];
+        partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * EN_NV + t] = s;
+    }
+}
+
+// res[b * S + v] = sum over the nblk partials [b][blk][S] (fixed order), v < nval
+template <int S>
+__global__ void __launch_bounds__(RED_THREADS) k_finish(const double *__restrict__ partials, int nblk, int nval,
+                                                       double *__restrict__ res) {
+    __shared__ double sh[RED_THREADS / 32][S];
+    const int b = blockIdx.x, t = threadIdx.x;
+    double acc[S];
+#pragma unroll
+    for (int v = 0; v < S; ++v) acc[v] = 0.0;
+    for (int k = t; k < nblk; k += RED_THREADS) {
+        const double *p = partials + ((long long)b * nblk + k) * S;
+#pragma unroll
+        for (int v = 0; v < S; ++v)
+            if (v < nval) acc[v] += p[v];
+    }
+#pragma unroll
+    for (int v = 0; v < S; ++v) {
+        const double x = warp_sum(acc[v]);
+        if ((t & 31) == 0) sh[t >> 5][v] = x;
+    }
+    __syncthreads();
+    if (t < nval) {
+        double s = 0.0;
+        for (int w = 0; w < RED_THREADS / 32; ++w) s += sh[w][t];
+        res[(long long)b * S + t] = s;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Density of states of Z~ = -sum_l sigma^z_l (Sec. V): weight of the amplitudes with k links
+// in sigma^z = -1.  Each thread keeps its own column of bins in shared memory (no atomics) and
+// adds one sum per number of links set among its register bits; complex64 weights are exact
+// products in two-float sums on the FP32 pipes.  partials[(b * gridDim.x + blk) * nbins + k].
+// 27 qubits in complex64 0.40 ms (one FP64 shared-memory atomic per amplitude: 12.5), 24 qubits
+// in complex128 0.09 (1.4).
+// ---------------------------------------------------------------------------
+template <typename R> struct Bin;
+template <> struct Bin<double> {
+    typedef double T;
+    static __device__ __forceinline__ T zero() { return 0.0; }
+    static __device__ __forceinline__ void weigh(T &s, double2 a) { s = fma(a.y, a.y, fma(a.x, a.x, s)); }
+    static __device__ __forceinline__ T sum(T a, T b) { return a + b; }
+    static __device__ __forceinline__ double value(T a) { return a; }
+};
+template <> struct Bin<float> {
+    typedef float2 T;      // high, low
+    static __device__ __forceinline__ T zero() { return make_float2(0.f, 0.f); }
+    static __device__ __forceinline__ void add(T &s, float x, float e) {
+        const float h = __fadd_rn(s.x, x), b = __fsub_rn(h, s.x);
+        s.y = __fadd_rn(s.y, __fadd_rn(e, __fadd_rn(__fsub_rn(s.x, __fsub_rn(h, b)), __fsub_rn(x, b))));
+        s.x = h;
+    }
+    static __device__ __forceinline__ void weigh(T &s, float2 a) {
+        const float p = __fmul_rn(a.x, a.x), q = __fmul_rn(a.y, a.y);
+        add(s, p, __fmaf_rn(a.x, a.x, -p));
+        add(s, q, __fmaf_rn(a.y, a.y, -q));
+    }
+    static __device__ __forceinline__ T sum(T a, T b) { add(a, b.x, b.y); return a; }
+    static __device__ __forceinline__ double value(T a) { return (double)a.x + (double)a.y; }
+};
+
+template <typename R>
+__global__ void __launch_bounds__(RED_THREADS) k_dos(const typename C2<R>::T *__restrict__ psi, int n,
+                                                    long long state_stride, unsigned long long linkmask, int nbins,
+                                                    double *__restrict__ partials) {
+    using V = typename C2<R>::T;
+    typedef Bin<R> B;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    typename B::T *bins = reinterpret_cast<typename B::T *>(smem_raw);     // [nbins][RED_THREADS]
+    const int t = threadIdx.x;
+    for (int k = 0; k < nbins; ++k) bins[k * RED_THREADS + t] = B::zero();
+    psi += (long long)blockIdx.y * state_stride;
+    const long long dim = 1ll << n, ntiles = n > LT ? dim >> LT : 1;
+    const unsigned reg = (unsigned)(linkmask >> TB) & 15u;                 // links among the register bits
+    const int kt = __popc(t & (unsigned)linkmask & 255u);
+    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const V *p0 = psi + (tile << LT) + t;
+        V v[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            v[r] = n >= LT || (r << TB) + t < dim ? p0[r << TB] : mk<R>((R)0, (R)0);
+        typename B::T *col = bins + (kt + __popcll(((unsigned long long)tile << LT) & linkmask)) * RED_THREADS + t;
+        if (reg == 15u || reg == 0u) {
+            typename B::T s[RB + 1];
+#pragma unroll
+            for (int k = 0; k <= RB; ++k) s[k] = B::zero();
+            if (reg) {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) B::weigh(s[(r & 1) + ((r >> 1) & 1) + ((r >> 2) & 1) + (r >> 3)], v[r]);
+#pragma unroll
+                for (int k = 0; k <= RB; ++k) col[k * RED_THREADS] = B::sum(col[k * RED_THREADS], s[k]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) B::weigh(s[0], v[r]);
+                col[0] = B::sum(col[0], s[0]);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                typename B::T s = B::zero();
+                B::weigh(s, v[r]);
+                typename B::T *c = col + __popc((unsigned)r & reg) * RED_THREADS;
+                *c = B::sum(*c, s);
+            }
+        }
+    }
+    __syncthreads();
+    for (int k = t >> 5; k < nbins; k += RED_THREADS / 32) {
+        double s = 0.0;
+        for (int j = t & 31; j < RED_THREADS; j += 32) s += B::value(bins[k * RED_THREADS + j]);
+        s = warp_sum(s);
+        if ((t & 31) == 0) partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * nbins + k] = s;
+    }
+}
+
+// out[b * nval + v] = sum over nblk partials (layout [b][blk][v]), one warp per value, fixed order
+__global__ void __launch_bounds__(1024) k_finish_wide(const double *__restrict__ partials, int nblk, int nval,
+                                                     double *__restrict__ out) {
+    const int b = blockIdx.x, lane = threadIdx.x & 31;
+    for (int v = threadIdx.x >> 5; v < nval; v += 32) {
+        double s = 0.0;
+        for (int k = lane; k < nblk; k += 32) s += partials[((long long)b * nblk + k) * nval + v];
+        s = warp_sum(s);
+        if (lane == 0) out[(long long)b * nval + v] = s;
+    }
+}
+
+}  // namespace qsim

@@ -18,6 +18,7 @@
 #include "qsim.h"
 #include "lattice.h"
 #include "kernels.cuh"
+#include "measure.cuh"
 #include "xpass_tma.cuh"
 #include "xpass_wl.cuh"
 #include "xpass_df.cuh"
@@ -805,27 +806,50 @@ qs_status run_op_pergate(qs_sim *s, const Op *ops_b) {
 // ---------------------------------------------------------------------------
 // reductions
 // ---------------------------------------------------------------------------
+// Blocks per state of a reduction over 4096-amplitude tiles.
+unsigned red_blocks(const qs_sim *s) {
+    return (unsigned)std::min<long long>(RED_BLOCKS, std::max<long long>(1, s->dim >> LT));
+}
+
+// norm into value 0; sums: the two diagonal sums into 1 and 2; zmask != 0: <Z_zmask> into 3
 template <typename R>
-qs_status reduce_diag(qs_sim *s, const void *state, uint64_t zmask, int slot) {
-    dim3 grid(RED_BLOCKS, (unsigned)s->batch);
-    k_reduce_diag<R><<<grid, RED_THREADS, 0, s->stream>>>((const V<R> *)state, s->n, s->dim, s->d_colA,
-                                                          s->d_colB, s->nA, s->nB,
-                                                          (unsigned long long)zmask, s->d_partials);
+qs_status reduce_diag(qs_sim *s, const void *state, uint64_t zmask, int slot, bool sums) {
+    const unsigned G = red_blocks(s);
+    auto kern = sums ? (zmask ? k_reduce_diag<R, true, true> : k_reduce_diag<R, true, false>)
+                     : (zmask ? k_reduce_diag<R, false, true> : k_reduce_diag<R, false, false>);
+    kern<<<dim3(G, (unsigned)s->batch), RED_THREADS, 0, s->stream>>>((const V<R> *)state, s->n, s->dim, s->d_colA,
+                                                                     s->d_colB, s->nA, s->nB,
+                                                                     (unsigned long long)zmask, s->d_partials);
     CKL(s); s->launches++;
-    k_finish<<<s->batch, RED_THREADS, 0, s->stream>>>(s->d_partials, RED_BLOCKS, 4,
-                                                      s->d_res + (size_t)slot * s->batch * RED_NV);
+    k_finish<RED_NV><<<s->batch, RED_THREADS, 0, s->stream>>>(s->d_partials, (int)G, 4,
+                                                              s->d_res + (size_t)slot * s->batch * RED_NV);
     CKL(s); s->launches++;
     return QS_OK;
 }
 
+// <a|b>
 template <typename R>
-qs_status reduce_xmask(qs_sim *s, const void *a, const void *b, uint64_t mask, int slot) {
-    dim3 grid(RED_BLOCKS, (unsigned)s->batch);
-    k_reduce_xmask<R><<<grid, RED_THREADS, 0, s->stream>>>((const V<R> *)a, (const V<R> *)b, s->n, s->dim,
-                                                           (unsigned long long)mask, s->d_partials);
+qs_status reduce_dot(qs_sim *s, const void *a, const void *b, int slot) {
+    const unsigned G = red_blocks(s);
+    k_reduce_dot<R><<<dim3(G, (unsigned)s->batch), RED_THREADS, 0, s->stream>>>((const V<R> *)a, (const V<R> *)b, s->n,
+                                                                                s->dim, s->d_partials);
     CKL(s); s->launches++;
-    k_finish<<<s->batch, RED_THREADS, 0, s->stream>>>(s->d_partials, RED_BLOCKS, 2,
-                                                      s->d_res + (size_t)slot * s->batch * RED_NV);
+    k_finish<RED_NV><<<s->batch, RED_THREADS, 0, s->stream>>>(s->d_partials, (int)G, 2,
+                                                              s->d_res + (size_t)slot * s->batch * RED_NV);
+    CKL(s); s->launches++;
+    return QS_OK;
+}
+
+// <X_mask> of the bound state
+template <typename R>
+qs_status reduce_xmask(qs_sim *s, uint64_t mask, int slot) {
+    if (mask == 0) return reduce_dot<R>(s, s->state[0], s->state[0], slot);
+    const unsigned G = red_blocks(s);
+    k_reduce_xpair<R><<<dim3(G, (unsigned)s->batch), RED_THREADS, 0, s->stream>>>(
+        (const V<R> *)s->state[0], s->n, s->dim, (unsigned long long)mask, 63 - __builtin_clzll(mask), s->d_partials);
+    CKL(s); s->launches++;
+    k_finish<RED_NV><<<s->batch, RED_THREADS, 0, s->stream>>>(s->d_partials, (int)G, 2,
+                                                              s->d_res + (size_t)slot * s->batch * RED_NV);
     CKL(s); s->launches++;
     return QS_OK;
 }
@@ -841,12 +865,14 @@ qs_status check_device_flag(qs_sim *s) {
     return QS_OK;
 }
 
+// The results and the error flag in one wait (the flag sits behind the results in h_res).
 qs_status read_results(qs_sim *s, int slots) {
     size_t bytes = (size_t)slots * s->batch * RED_NV * sizeof(double);
+    int *flag = reinterpret_cast<int *>(s->h_res + (size_t)RES_SLOTS * s->batch * RED_NV);
     CK(s, cudaMemcpyAsync(s->h_res, s->d_res, bytes, cudaMemcpyDeviceToHost, s->stream));
+    CK(s, cudaMemcpyAsync(flag, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
     CK(s, cudaStreamSynchronize(s->stream));
-    qs_status st = check_device_flag(s);
-    if (st != QS_OK) return st;
+    if (*flag) return check_device_flag(s);
     for (size_t i = 0; i < (size_t)slots * s->batch * RED_NV; ++i)
         if (!std::isfinite(s->h_res[i])) FAIL(s, QS_ERR_NONFINITE, "non-finite reduction result");
     return QS_OK;
@@ -864,7 +890,7 @@ qs_status renormalise(qs_sim *s) {
         if ((st = renormalise<R>(s)) != QS_OK) return st;
         return df_convert(s, true);
     }
-    if ((st = reduce_diag<R>(s, s->state[0], 0, 0)) != QS_OK) return st;
+    if ((st = reduce_diag<R>(s, s->state[0], 0, 0, false)) != QS_OK) return st;
     dim3 grid(152 * 8, (unsigned)s->batch);
     k_scale_by_norm<R><<<grid, 256, 0, s->stream>>>((V<R> *)s->state[0], s->dim, s->d_res);
     CKL(s); s->launches++;
@@ -1314,10 +1340,10 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
             CKL(s); s->launches++;
         }
         CK(s, cudaStreamSynchronize(s->stream));   // h is a host temporary
-        if ((st = reduce_xmask<R>(s, psi, lam, 0, 0)) != QS_OK) return st;   // <psi|H1|psi>
+        if ((st = reduce_dot<R>(s, psi, lam, 0)) != QS_OK) return st;   // <psi|H1|psi>
     } else {
         if (!ref) FAIL(s, QS_ERR_ARG, "fidelity target needs a reference state");
-        if ((st = reduce_xmask<R>(s, ref, psi, 0, 0)) != QS_OK) return st;   // <phi|psi>
+        if ((st = reduce_dot<R>(s, ref, psi, 0)) != QS_OK) return st;   // <phi|psi>
         k_scaled_copy<R><<<dim3(152 * 8, B), 256, 0, s->stream>>>(lam, (const V<R> *)ref, s->dim, s->d_res);
         CKL(s); s->launches++;
     }
@@ -1433,7 +1459,7 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
             }
             if (done[0] != s->nX0 || done[1] != s->nX1)
                 FAIL(s, QS_ERR_STATE, "reverse passes do not cover every X qubit once");
-            k_finish<<<B, RED_THREADS, 0, s->stream>>>(part_j, (int)nblk_t, 4, s->d_grad + jj * B * RED_NV);
+            k_finish<RED_NV><<<B, RED_THREADS, 0, s->stream>>>(part_j, (int)nblk_t, 4, s->d_grad + jj * B * RED_NV);
             CKL(s); s->launches++;
             carried = next_carried;
             continue;
@@ -1445,7 +1471,7 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
                                                                s->d_adj_part, (int)nblk, pi * (int)G);
             CKL(s); s->launches++;
         }
-        k_finish<<<B, RED_THREADS, 0, s->stream>>>(s->d_adj_part, (int)nblk, 4, s->d_grad + jj * B * RED_NV);
+        k_finish<RED_NV><<<B, RED_THREADS, 0, s->stream>>>(s->d_adj_part, (int)nblk, 4, s->d_grad + jj * B * RED_NV);
         CKL(s); s->launches++;
     }
     CK(s, cudaMemcpyAsync(s->h_grad, s->d_grad, nops * B * RED_NV * sizeof(double), cudaMemcpyDeviceToHost,
@@ -1580,7 +1606,8 @@ qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch
     size_t rbytes = (size_t)RES_SLOTS * batch * RED_NV * sizeof(double);
     if (cudaMalloc((void **)&s->d_partials, pbytes) != cudaSuccess) return fail("partials");
     if (cudaMalloc((void **)&s->d_res, rbytes) != cudaSuccess) return fail("results");
-    if (cudaMallocHost((void **)&s->h_res, rbytes) != cudaSuccess) return fail("pinned results");
+    if (cudaMemset(s->d_res, 0, rbytes) != cudaSuccess) return fail("results");
+    if (cudaMallocHost((void **)&s->h_res, rbytes + sizeof(double)) != cudaSuccess) return fail("pinned results");
     if (cudaEventCreateWithFlags(&s->rec_done, cudaEventDisableTiming) != cudaSuccess) return fail("event");
     if (cudaMalloc((void **)&s->d_err, sizeof(int)) != cudaSuccess) return fail("error flag");
     if (cudaMemset(s->d_err, 0, sizeof(int)) != cudaSuccess) return fail("error flag");
@@ -1612,7 +1639,9 @@ qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch
         cudaFuncSetAttribute(k_adj_xpass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
         cudaFuncSetAttribute(k_apply_h_pass<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
         cudaFuncSetAttribute(k_apply_h_pass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
-        cudaFuncSetAttribute(k_xmeasure<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)((1 << LT) * 16));
+        cudaFuncSetAttribute(k_energy<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)((1 << LT) * 16));
+        cudaFuncSetAttribute(k_dos<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * RED_THREADS * 8);
+        cudaFuncSetAttribute(k_dos<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * RED_THREADS * 8);
         for (int v = 0; v < 3; ++v) {
             const bool tn = v >= 1, mg = v == 2;
             cudaFuncSetAttribute(adj_tma_kernel(2, tn, mg), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1833,15 +1862,57 @@ qs_status qs_evolve(qs_sim *s, const qs_couplings *c, const double *sv, double d
 
 }  // extern "C"
 
+// Every term of <H>: per state EN_NV values [norm, sum Z_A, sum Z_B, sum X class 0, class 1] at
+// h_res[b * EN_NV] (one launch and the sum over its blocks; synchronises).
+template <typename R>
+static qs_status energy_terms(qs_sim *s) {
+    qs_status st;
+    const int B = s->batch;
+    EnergyParams P;
+    memset(&P, 0, sizeof(P));
+    P.n = s->n; P.nA = s->nA; P.nB = s->nB;
+    // twelve qubits, then eight per pass (whatever the plan of the evolution)
+    for (int next = 0; s->n >= LT && next < s->n; ++P.np) {
+        const int k = next ? std::min(8, s->n - next) : 0;
+        P.c[P.np] = LT - k;
+        P.next[P.np] = next ? next : LT;
+        P.k[P.np] = k;
+        next = next ? next + k : LT;
+    }
+    const int np = P.np;
+    for (int q = 0; q < s->n; ++q) {
+        if (s->lat.x_class[q]) P.cls |= 1ull << q;
+        if (np == 0) {
+            if (s->lat.x_class[q]) P.mask_cls |= 1ull << P.nmasks;
+            P.mask[P.nmasks++] = 1ull << q;
+        }
+    }
+    if (!s->lat.gauge_higgs)
+        for (uint64_t m : s->lat.stars) {
+            P.mask_cls |= 1ull << P.nmasks;
+            P.mask[P.nmasks++] = m;
+        }
+    const long long ntiles = std::max<long long>(1, s->dim >> LT);
+    P.gp = (int)std::min<long long>(ntiles, (long long)s->sm_count * (sizeof(R) == 4 ? 3 : 2));
+    P.gm = P.nmasks ? (int)std::min<long long>(ntiles, (long long)s->sm_count * 4) : 0;
+    const size_t nblk = (size_t)np * P.gp + P.gm;
+    if ((st = grow(s, &s->d_adj_part, &s->adj_part_cap, nblk * B * EN_NV, false)) != QS_OK) return st;
+    k_energy<R><<<dim3((unsigned)nblk, B), NT, np ? (size_t)(1 << LT) * sizeof(V<R>) : 0, s->stream>>>(
+        (const V<R> *)s->state[0], s->dim, s->d_colA, s->d_colB, P, s->d_adj_part);
+    CKL(s); s->launches++;
+    k_finish<EN_NV><<<B, RED_THREADS, 0, s->stream>>>(s->d_adj_part, (int)nblk, EN_NV, s->d_res);
+    CKL(s); s->launches++;
+    return read_results(s, EN_NV / RED_NV);
+}
+
 template <typename R>
 static qs_status expect_impl(qs_sim *s, int kind, int index, const qs_couplings *c, double sval, double *out) {
     qs_status st;
     const Lattice &L = s->lat;
     const int B = s->batch;
-    auto xm = [&](uint64_t m, int slot) { return reduce_xmask<R>(s, s->state[0], s->state[0], m, slot); };
     switch (kind) {
         case QS_NORM:
-            if ((st = reduce_diag<R>(s, s->state[0], 0, 0)) != QS_OK) return st;
+            if ((st = reduce_diag<R>(s, s->state[0], 0, 0, false)) != QS_OK) return st;
             if ((st = read_results(s, 1)) != QS_OK) return st;
             for (int b = 0; b < B; ++b) out[b] = res(s, 0, b, 0);
             return QS_OK;
@@ -1855,10 +1926,11 @@ static qs_status expect_impl(qs_sim *s, int kind, int index, const qs_couplings 
                 if (index < 0 || index >= (int)L.wilson.size()) FAIL(s, QS_ERR_ARG, "Wilson loop index");
                 m = L.wilson[index];
             }
-            if ((st = reduce_diag<R>(s, s->state[0], m, 0)) != QS_OK) return st;
+            const bool mean = kind == QS_PLAQUETTE && index == -1;
+            if ((st = reduce_diag<R>(s, s->state[0], m, 0, mean)) != QS_OK) return st;
             if ((st = read_results(s, 1)) != QS_OK) return st;
             for (int b = 0; b < B; ++b)
-                out[b] = (kind == QS_PLAQUETTE && index == -1) ? res(s, 0, b, 1) / L.plaquettes.size()
+                out[b] = mean ? res(s, 0, b, 1) / L.plaquettes.size()
                                                                : res(s, 0, b, 3);
             return QS_OK;
         }
@@ -1876,7 +1948,7 @@ static qs_status expect_impl(qs_sim *s, int kind, int index, const qs_couplings 
                 if (index < 0 || index >= (int)L.thooft.size()) FAIL(s, QS_ERR_ARG, "'t Hooft index");
                 m = L.thooft[index];
             }
-            if ((st = xm(m, 0)) != QS_OK) return st;
+            if ((st = reduce_xmask<R>(s, m, 0)) != QS_OK) return st;
             if ((st = read_results(s, 1)) != QS_OK) return st;
             for (int b = 0; b < B; ++b) out[b] = res(s, 0, b, 0);
             return QS_OK;
@@ -1885,49 +1957,11 @@ static qs_status expect_impl(qs_sim *s, int kind, int index, const qs_couplings 
         case QS_ENERGY_S: {
             if (!c) FAIL(s, QS_ERR_ARG, "energy needs couplings");
             double sv = (kind == QS_ENERGY) ? 1.0 : sval;
-            int slot = 0;
-            if ((st = reduce_diag<R>(s, s->state[0], 0, slot++)) != QS_OK) return st;
-            const int np = (int)s->passes.size();
-            int xslot = -1;
-            if (np > 0) {
-                // single-qubit X terms: one read-only sweep per pass, sums per class
-                const long long ntiles = 1ll << (s->n - LT);
-                const unsigned G = (unsigned)std::min<long long>(ntiles, (long long)s->sm_count * 4);
-                const size_t nblk = (size_t)np * G;
-                if ((st = grow(s, &s->d_adj_part, &s->adj_part_cap, nblk * B * RED_NV, false)) != QS_OK) return st;
-                const size_t smem = (size_t)(1 << LT) * sizeof(V<R>);
-                for (int p = 0; p < np; ++p) {
-                    k_xmeasure<R><<<dim3(G, B), NT, smem, s->stream>>>((const V<R> *)s->state[0], s->dim, ntiles,
-                                                                      s->d_passes + NVAR * p, s->d_adj_part,
-                                                                      (int)nblk, p * (int)G);
-                    CKL(s); s->launches++;
-                }
-                xslot = slot++;
-                k_finish<<<B, RED_THREADS, 0, s->stream>>>(s->d_adj_part, (int)nblk, 2,
-                                                           s->d_res + (size_t)xslot * B * RED_NV);
-                CKL(s); s->launches++;
-            }
-            const int q0 = slot;
-            if (np == 0)
-                for (int q = 0; q < s->n; ++q)
-                    if ((st = xm(1ull << q, slot++)) != QS_OK) return st;
-            int star0 = slot;
-            if (!L.gauge_higgs)
-                for (uint64_t m : L.stars)
-                    if ((st = xm(m, slot++)) != QS_OK) return st;
-            if ((st = read_results(s, slot)) != QS_OK) return st;
+            if ((st = energy_terms<R>(s)) != QS_OK) return st;
             for (int b = 0; b < B; ++b) {
-                Coef q = coefficients(c[b], sv);
-                double e = -q.za * res(s, 0, b, 1) - q.zb * res(s, 0, b, 2);
-                if (xslot >= 0) {
-                    // each pair counted once: <X_q> = 2 sum_pairs Re(conj(a) b)
-                    e -= q.xs * 2.0 * res(s, xslot, b, 0) + q.xt * 2.0 * res(s, xslot, b, 1);
-                } else {
-                    for (int k = 0; k < s->n; ++k)
-                        e -= (L.x_class[k] ? q.xt : q.xs) * res(s, q0 + k, b, 0);
-                }
-                for (int k = star0; k < slot; ++k) e -= q.xt * res(s, k, b, 0);
-                out[b] = e;
+                const Coef q = coefficients(c[b], sv);
+                const double *v = s->h_res + (size_t)b * EN_NV;
+                out[b] = -q.za * v[1] - q.zb * v[2] - q.xs * v[3] - q.xt * v[4];
             }
             return QS_OK;
         }
@@ -1953,15 +1987,14 @@ qs_status qs_expect_pauli(qs_sim *s, int type, uint64_t mask, double *out) {
     if (type != 0 && type != 1) FAIL(s, QS_ERR_ARG, "type must be 0 (Z) or 1 (X)");
     if (s->n < 64 && (mask >> s->n) != 0) FAIL(s, QS_ERR_ARG, "mask has bits beyond the qubit count");
     if (type == 0) {
-        st = s->dtype == QS_C64 ? reduce_diag<float>(s, s->state[0], mask, 0)
-                                : reduce_diag<double>(s, s->state[0], mask, 0);
+        st = s->dtype == QS_C64 ? reduce_diag<float>(s, s->state[0], mask, 0, false)
+                                : reduce_diag<double>(s, s->state[0], mask, 0, false);
     } else {
-        st = s->dtype == QS_C64 ? reduce_xmask<float>(s, s->state[0], s->state[0], mask, 0)
-                                : reduce_xmask<double>(s, s->state[0], s->state[0], mask, 0);
+        st = s->dtype == QS_C64 ? reduce_xmask<float>(s, mask, 0) : reduce_xmask<double>(s, mask, 0);
     }
     if (st != QS_OK) return st;
     if ((st = read_results(s, 1)) != QS_OK) return st;
-    for (int b = 0; b < s->batch; ++b) out[b] = res(s, 0, b, type == 0 ? 3 : 0);
+    for (int b = 0; b < s->batch; ++b) out[b] = res(s, 0, b, type == 0 && mask ? 3 : 0);
     return QS_OK;
 }
 
@@ -1969,8 +2002,7 @@ qs_status qs_fidelity(qs_sim *s, const void *ref, double *out) {
     qs_status st;
     if ((st = check_ready(s)) != QS_OK) return st;
     if (!ref || !out) FAIL(s, QS_ERR_ARG, "null argument");
-    st = s->dtype == QS_C64 ? reduce_xmask<float>(s, ref, s->state[0], 0, 0)
-                            : reduce_xmask<double>(s, ref, s->state[0], 0, 0);
+    st = s->dtype == QS_C64 ? reduce_dot<float>(s, ref, s->state[0], 0) : reduce_dot<double>(s, ref, s->state[0], 0);
     if (st != QS_OK) return st;
     if ((st = read_results(s, 1)) != QS_OK) return st;
     for (int b = 0; b < s->batch; ++b) {
@@ -2081,10 +2113,20 @@ qs_status qs_scan(qs_sim *s, const qs_couplings *points, int n_points, const dou
         auto put = [&](int k, const double *v) {
             for (int b = 0; b < cnt; ++b) out[(size_t)(p0 + b) * SCAN_NOBS + k] = v[b];
         };
-        if ((st = qs_expect(s, QS_ENERGY, 0, chunk.data(), 1.0, tmp.data())) != QS_OK) return st;
-        put(0, tmp.data());
-        if ((st = qs_expect(s, QS_PLAQUETTE, -1, nullptr, 1.0, tmp.data())) != QS_OK) return st;
-        put(1, tmp.data());
+        // energy, mean plaquette, norm and the mean fields from the terms of one measurement
+        if ((st = s->dtype == QS_C64 ? energy_terms<float>(s) : energy_terms<double>(s)) != QS_OK) return st;
+        const int nl = s->lat.n_links, nv = s->n - s->lat.n_links;
+        for (int b = 0; b < cnt; ++b) {
+            const Coef q = coefficients(chunk[b], 1.0);
+            const double *v = s->h_res + (size_t)b * EN_NV;
+            double *o = out + (size_t)(p0 + b) * SCAN_NOBS;
+            o[0] = -q.za * v[1] - q.zb * v[2] - q.xs * v[3] - q.xt * v[4];
+            o[1] = v[1] / s->lat.plaquettes.size();
+            o[4] = v[0];
+            o[5] = nl ? v[3] / nl : 0.0;
+            o[6] = nv ? v[4] / nv : 0.0;
+            o[7] = 0.0;
+        }
         for (int w = 0; w < 2; ++w) {
             if (w < (int)s->lat.wilson.size()) {
                 if ((st = qs_expect(s, QS_WILSON, w, nullptr, 1.0, tmp.data())) != QS_OK) return st;
@@ -2093,20 +2135,6 @@ qs_status qs_scan(qs_sim *s, const qs_couplings *points, int n_points, const dou
             }
             put(2 + w, tmp.data());
         }
-        if ((st = qs_expect(s, QS_NORM, 0, nullptr, 1.0, tmp.data())) != QS_OK) return st;
-        put(4, tmp.data());
-        // link / vertex <X> averages
-        std::vector<double> xs(B, 0.0), xt(B, 0.0);
-        for (int q = 0; q < s->n; ++q) {
-            if ((st = qs_expect(s, QS_X, q, nullptr, 1.0, tmp.data())) != QS_OK) return st;
-            for (int b = 0; b < B; ++b) (s->lat.x_class[q] ? xt : xs)[b] += tmp[b];
-        }
-        const int nl = s->lat.n_links, nv = s->n - s->lat.n_links;
-        for (int b = 0; b < B; ++b) { xs[b] = nl ? xs[b] / nl : 0.0; xt[b] = nv ? xt[b] / nv : 0.0; }
-        put(5, xs.data());
-        put(6, xt.data());
-        std::fill(tmp.begin(), tmp.end(), 0.0);
-        put(7, tmp.data());
     }
     return QS_OK;
 }
@@ -2121,18 +2149,19 @@ qs_status qs_dos(qs_sim *s, double *out) {
     if (nbins > 64) FAIL(s, QS_ERR_ARG, "too many links");
     uint64_t linkmask = 0;
     for (int q = 0; q < s->n; ++q) if (!s->lat.x_class[q]) linkmask |= 1ull << q;
-    const int G = 152 * 4;
+    const int G = (int)red_blocks(s);
+    const size_t bins = (size_t)nbins * RED_THREADS * 8;
     if ((st = grow(s, &s->d_adj_part, &s->adj_part_cap, (size_t)G * B * nbins + (size_t)B * nbins, false)) != QS_OK)
         return st;
     double *dout = s->d_adj_part + (size_t)G * B * nbins;
     if (s->dtype == QS_C64)
-        k_dos<float><<<dim3(G, B), RED_THREADS, 0, s->stream>>>((const float2 *)s->state[0], s->n, s->dim, linkmask,
+        k_dos<float><<<dim3(G, B), RED_THREADS, bins, s->stream>>>((const float2 *)s->state[0], s->n, s->dim, linkmask,
                                                                 nbins, s->d_adj_part);
     else
-        k_dos<double><<<dim3(G, B), RED_THREADS, 0, s->stream>>>((const double2 *)s->state[0], s->n, s->dim,
+        k_dos<double><<<dim3(G, B), RED_THREADS, bins, s->stream>>>((const double2 *)s->state[0], s->n, s->dim,
                                                                  linkmask, nbins, s->d_adj_part);
     CKL(s); s->launches++;
-    k_finish_wide<<<B, 64, 0, s->stream>>>(s->d_adj_part, G, nbins, dout);
+    k_finish_wide<<<B, 1024, 0, s->stream>>>(s->d_adj_part, G, nbins, dout);
     CKL(s); s->launches++;
     CK(s, cudaMemcpyAsync(out, dout, (size_t)B * nbins * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     CK(s, cudaStreamSynchronize(s->stream));
