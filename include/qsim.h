@@ -133,7 +133,10 @@ typedef enum {
                                  fusing k new qubits keeps a contiguous chunk of 12 - k
                                  low qubits, 2^(12-k) amplitudes per row); 0 (default):
                                  8 per pass, the remainder last.  Rejected (QS_ERR_ARG)
-                                 for states of fewer than 13 qubits.                  */
+                                 for states of fewer than 13 qubits.  With the default
+                                 plan, complex64 unitary-gauge runs of one state may use
+                                 larger tiles (13 qubits, then up to 10 per pass) where
+                                 they save passes: 21 to 23 and 29 to 33 qubits.       */
     QS_OPT_SCAN_BUFFERS = 12, /* qs_scan_mixed: 32 KB tile buffers per CTA of the
                                  larger lattice's passes, 2 or 3 (two CTAs per SM) or 4
                                  or 6 (one CTA per SM; a pass keeps buffers - 1 loads in
@@ -147,7 +150,8 @@ typedef enum {
                                  slices of a tile through both rounds with warp-level
                                  synchronisation only, one thread issues the TMA
                                  copies over pooled tile buffers; 0: the CTA-staged
-                                 kernels                                              */
+                                 kernels.  Setting it, to either, also keeps the tiles
+                                 of 12 qubits that these kernels run on (QS_OPT_PLAN)  */
     QS_OPT_C128_DF = 14       /* complex128, unitary gauge, fused kernels: 1 (default):
                                  the Walsh-Hadamard passes run in double-float
                                  arithmetic (each real number an unevaluated sum of two

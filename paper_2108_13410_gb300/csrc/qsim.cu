@@ -5,6 +5,7 @@
 // sequencing on the bound stream, and FP64 reductions read back to the host.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <functional>
 #include <cstdio>
@@ -22,6 +23,7 @@
 #include "xpass_tma.cuh"
 #include "xpass_wl.cuh"
 #include "xpass_df.cuh"
+#include "xpass_wide.cuh"
 #include "adjoint.cuh"
 #include "adjoint_tma.cuh"
 #include "adjoint_wl.cuh"
@@ -100,11 +102,16 @@ struct qs_sim {
     int xmerge = 1;                        // share the pass of one qubit group between factor groups
     int pdl = 1;                           // X passes launched with programmatic stream serialisation
     int nbuf_shared = 0;                   // TMA tile buffers of the shared passes (0 auto, 2 or 3)
+    bool shared_kernel_set = false;        // QS_OPT_SHARED_KERNEL was set by the caller
     int shared_kernel = 1;                 // shared rotation passes: 1 warp-local slices where they
                                            // apply (k_xpass_wl), 0 the CTA-staged kernel
     int tan_off = 0;                       // tangent triple in the operator record
     int nX0 = 0, nX1 = 0;                  // X qubits per class
     bool tan_active = false;               // this call's X passes use the tangent form
+    // unitary gauge, complex64: passes over 2^13 tiles where they save passes (xpass_wide.cuh)
+    std::vector<WidePass> wide;            // [3 * pass + variant: H, H X, H Z]; empty: no saving
+    std::vector<int> wide_c, wide_w, wide_kw;   // chunk, first qubit and size of each pass's window
+    std::vector<CUtensorMap> wide_maps;
     // small states: the whole run of factor groups in one launch (resident.cu)
     ResParams res;
     int res_known = 0;                     // 0 not looked at yet, 1 the state fits, -1 it does not
@@ -329,6 +336,59 @@ void build_tma_passes(qs_sim *s) {
     }
 }
 
+// Passes over 2^13 tiles: 13 qubits, then windows of 9 or 10 qubits above a chunk of 4 or 3 (a
+// window of 9 may start on qubits that are already done).  Only where they are fewer than the
+// passes of 2^12 tiles: 21 to 23 and 29 to 33 qubits.  4x4 torus (32 qubits, 32 GiB): 4 passes
+// per step instead of 6.
+void build_wide_passes(qs_sim *s) {
+    s->wide.clear();
+    s->wide_c.clear(); s->wide_w.clear(); s->wide_kw.clear();
+    const int n = s->n, left = n - WT;
+    if (s->dtype != QS_C64 || s->lat.gauge_higgs || s->batch != 1 || left < 8) return;
+    const int np = 1 + (left + 9) / 10;
+    if (np >= 1 + (n - LT + 7) / 8 || np > 3) return;
+    int start = WT;
+    for (int p = 0; p < np; ++p) {
+        const int k = p == 0 ? 0 : np == 2 ? left : p == 1 ? (left <= 18 ? 9 : 10) : left - (left <= 18 ? 9 : 10);
+        const int kw = p == 0 ? 0 : std::max(9, k), w = start + k - kw, c = WT - kw;
+        auto g = [&](int j) { return p == 0 || j < c ? j : w + (j - c); };
+        WidePass P;
+        memset(&P, 0, sizeof(P));
+        P.first = p == 0;
+        P.chunk = c;
+        for (int j = 0; j < WT; ++j)
+            if (p == 0 || g(j) >= start) P.mask |= 1u << j;
+        P.mid_bits = p ? w - c : 0;
+        P.tile_bits = n - WT;
+        P.total_tiles = 1 << (n - WT);
+        s->wide_c.push_back(c); s->wide_w.push_back(w); s->wide_kw.push_back(kw);
+        for (int v = 0; v < 3; ++v) {
+            WidePass Q = P;
+            const PassDesc &d = s->pvar[v == 1 ? V_HAD_X : V_HAD_Z];   // table geometry and columns
+            Q.diag = v != 0;
+            Q.nA = d.nA; Q.nB = d.nB; Q.lut_off = d.lut_off;
+            Q.scale = v == 1 ? (float)d.scale : 1.0f;
+            const bool c3 = p && c == 3;
+            for (int j = 0; j < 8; ++j) {
+                const int q = g(c3 ? (j < 3 ? j : j + 5) : j < 4 ? j : j + 4);
+                Q.pa_thr[j] = d.colA[q]; Q.pb_thr[j] = d.colB[q];
+            }
+            for (int r = 0; r < WR; ++r)
+                for (int k2 = 0; k2 < 5; ++k2)
+                    if ((r >> k2) & 1) {
+                        const int q = g(c3 ? 3 + k2 : k2 < 4 ? 4 + k2 : 12);
+                        Q.pa_reg[r] ^= d.colA[q]; Q.pb_reg[r] ^= d.colB[q];
+                    }
+            for (int i = 0; i < Q.tile_bits; ++i) {
+                const int q = p == 0 ? WT + i : i < Q.mid_bits ? c + i : w + kw + (i - Q.mid_bits);
+                Q.pa_tile[i] = d.colA[q]; Q.pb_tile[i] = d.colB[q];
+            }
+            s->wide.push_back(Q);
+        }
+        start += p == 0 ? 0 : k;
+    }
+}
+
 // Encode one 5-D tensor map per pass over the bound complex64 state:
 //   dims (8-byte elements) {16, 2^(c-4), 2^(next-c), 2^k, 2^(n-next-k) * batch},
 //   box {16, 2^(c-4), 1, 2^k, 1}, 128-byte swizzle.
@@ -337,6 +397,7 @@ qs_status encode_tmaps(qs_sim *s, int slot = 0) {
     bool &ok = slot == 0 ? s->tmaps_ok : s->tmaps_aux_ok;
     ok = false;
     maps.clear();
+    if (slot == 0) s->wide_maps.clear();
     if (slot == 0) { s->tmaps_df_ok = false; s->tmaps_dfh.clear(); s->tmaps_dfl.clear(); }
     if (s->passes.empty() || !s->state[slot]) return QS_OK;
     if (s->dtype != QS_C64 && !(s->dtype == QS_C128 && slot == 0)) return QS_OK;
@@ -387,6 +448,24 @@ qs_status encode_tmaps(qs_sim *s, int slot = 0) {
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) FAIL(s, QS_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d) for pass %zu", (int)r, p);
         maps.push_back(m);
+    }
+    for (size_t p = 0; slot == 0 && p < s->wide_c.size(); ++p) {
+        const int c = s->wide_c[p], w = s->wide_w[p], kw = s->wide_kw[p];
+        const int ka = 5, kb = kw - ka;     // a box dimension holds at most 256 elements
+        cuuint64_t fd[5] = {16, 32, 16, 1ull << (n - WT), 1};
+        cuuint64_t fs[4] = {16 * 8, 512 * 8, 8192 * 8, (1ull << n) * 8};
+        cuuint32_t fb[5] = {16, 32, 16, 1, 1};
+        cuuint64_t wd[5] = {1ull << c, 1ull << (w - c), 1ull << ka, 1ull << (p ? kb : 0), 1ull << (n - w - kw)};
+        cuuint64_t ws[4] = {(1ull << c) * 8, (1ull << w) * 8, (1ull << (w + ka)) * 8, (1ull << (w + kw)) * 8};
+        cuuint32_t wb[5] = {1u << c, 1, 1u << ka, 1u << (p ? kb : 0), 1};
+        cuuint32_t es[5] = {1, 1, 1, 1, 1};
+        CUtensorMap m;
+        CUresult r = encode(&m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 5, s->state[slot], p ? wd : fd, p ? ws : fs, p ? wb : fb, es,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            p && c == 3 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) FAIL(s, QS_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d) for wide pass %zu", (int)r, p);
+        s->wide_maps.push_back(m);
     }
     ok = true;
     return QS_OK;
@@ -585,6 +664,55 @@ qs_status launch_xpass_df(qs_sim *s, int p, int variant, const double *rec, cons
     CKL(s);
     s->launches++;
     if (s->profile) CK(s, cudaEventRecord(e1, s->stream));
+    return QS_OK;
+}
+
+// CUDA events around a pass launch (QS_OPT_PROFILE): begin before it, *end recorded after it.
+qs_status profile_begin(qs_sim *s, bool merged, cudaEvent_t *end) {
+    *end = nullptr;
+    if (!s->profile) return QS_OK;
+    while (s->ev_pool.size() < s->ev_used + 2) {
+        cudaEvent_t e;
+        CK(s, cudaEventCreate(&e));
+        s->ev_pool.push_back(e);
+    }
+    CK(s, cudaEventRecord(s->ev_pool[s->ev_used], s->stream));
+    *end = s->ev_pool[s->ev_used + 1];
+    s->ev_used += 2;
+    s->ev_kind.resize(s->ev_used / 2);
+    s->ev_kind.back() = merged ? 1 : 0;
+    return QS_OK;
+}
+
+constexpr int W_SLICE_WARPS = 14;   // (15 the same, 18.7 instead of 18.5 ms with a chunk of three)
+
+size_t wide_smem_bytes(const qs_sim *s) {
+    return (size_t)W_NBUF * W_TILE_BYTES + 1024 + (size_t)s->max_lut * 8 + 3 * 256 * 8;
+}
+
+// One pass over 2^13 tiles; variant 0 H, 1 H and the X table, 2 H and the Z table; merged: H again.
+qs_status launch_xpass_wide(qs_sim *s, int p, int variant, const double *rec, bool merged) {
+    WidePass P = s->wide[3 * p + variant];
+    P.round2 = merged ? 1 : 0;
+    cudaEvent_t end;
+    qs_status st = profile_begin(s, merged, &end);
+    if (st != QS_OK) return st;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min(P.total_tiles, s->sm_count));
+    const auto kern = P.first ? k_xpass_wide<W_GROUPS, 16> : P.chunk == 4 ? k_xpass_wide<W_SLICE4, W_SLICE_WARPS>
+                                                                         : k_xpass_wide<W_SLICE3, W_SLICE_WARPS>;
+    cfg.blockDim = dim3(32 * ((P.first ? 16 : W_SLICE_WARPS) + 1));
+    cfg.dynamicSmemBytes = wide_smem_bytes(s);
+    cfg.stream = s->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = s->pdl ? 1 : 0;
+    CK(s, cudaLaunchKernelEx(&cfg, kern, rec, s->d_err, s->wide_maps[p], P));
+    CKL(s);
+    s->launches++;
+    if (end) CK(s, cudaEventRecord(end, s->stream));
     return QS_OK;
 }
 
@@ -1058,6 +1186,22 @@ qs_status launch_ops_merged(qs_sim *s, const std::vector<Op> &ops, int steps_per
     return QS_OK;
 }
 
+// 8 new qubits per pass, the remainder last
+bool default_plan(const qs_sim *s, const std::vector<int> &k) {
+    int left = s->n - LT;
+    for (int x : k) {
+        if (x != std::min(8, left)) return false;
+        left -= x;
+    }
+    return true;
+}
+
+// 2^13 tiles: by default (no kernel, plan or buffer option set) where they save passes.
+bool wide_schedule(const qs_sim *s) {
+    return !s->wide_maps.empty() && s->xpass_impl == 0 && s->plan_code == 0 && !s->shared_kernel_set &&
+           s->shared_kernel == 1 && s->nbuf_shared == 0 && s->tma_store;
+}
+
 // Unitary gauge with shared passes: the X layer of factor group k is H^n D_X H^n
 // (unnormalised Walsh-Hadamard passes around the Hadamard-basis phase table D_X) and
 // the Z layer is diagonal.  The D_X pass applies H(gx) D_X H(gx) on one qubit group, and
@@ -1071,22 +1215,27 @@ qs_status launch_ops_merged_ug(qs_sim *s, const std::vector<Op> &ops, int steps_
     qs_status st;
     const int B = s->batch;
     const size_t nops = ops.size() / B;
-    const int np = (int)s->passes.size();
+    const bool wide = sizeof(R) == 4 && wide_schedule(s);
+    const int np = wide ? (int)s->wide_maps.size() : (int)s->passes.size();
     const size_t rs = (size_t)B * s->rec_stride;
     const int gx = np - 1, gz = np - 2;
+    auto pass = [&](int p, int variant, const double *rec, const double *rec2 = nullptr) {
+        if (wide) return launch_xpass_wide(s, p, variant == V_HAD ? 0 : variant == V_HAD_X ? 1 : 2, rec, rec2 != nullptr);
+        return launch_xpass<R>(s, p, variant, rec, 0, rec2);
+    };
     bool carried = false;   // H(gz) of op k was applied by op k-1's Z pass
     for (size_t k = j0; k < j1; ++k) {
         const double *rec = s->d_rec + (k - j0) * rs;
         const bool has_z = ops[k * B].has_z;
-        if (!carried && (st = launch_xpass<R>(s, gz, V_HAD, rec)) != QS_OK) return st;
+        if (!carried && (st = pass(gz, V_HAD, rec)) != QS_OK) return st;
         for (int p = 0; p < np - 2; ++p)
-            if ((st = launch_xpass<R>(s, p, V_HAD, rec)) != QS_OK) return st;
-        if ((st = launch_xpass<R>(s, gx, V_HAD_X, rec, 0, rec)) != QS_OK) return st;   // H D_X H
+            if ((st = pass(p, V_HAD, rec)) != QS_OK) return st;
+        if ((st = pass(gx, V_HAD_X, rec, rec)) != QS_OK) return st;   // H D_X H
         for (int p = np - 3; p >= 0; --p)
-            if ((st = launch_xpass<R>(s, p, V_HAD, rec)) != QS_OK) return st;
+            if ((st = pass(p, V_HAD, rec)) != QS_OK) return st;
         carried = has_z && k + 1 < j1;
-        if (carried) st = launch_xpass<R>(s, gz, V_HAD_Z, rec, 0, rec + rs);      // H Z_k H(next)
-        else st = launch_xpass<R>(s, gz, has_z ? V_HAD_Z : V_HAD, rec);
+        if (carried) st = pass(gz, V_HAD_Z, rec, rec + rs);      // H Z_k H(next)
+        else st = pass(gz, has_z ? V_HAD_Z : V_HAD, rec);
         if (st != QS_OK) return st;
         if (s->renorm_every > 0 && steps_per_renorm_unit > 0 &&
             ((k + 1) % ((size_t)s->renorm_every * steps_per_renorm_unit) == 0 || k + 1 == nops))
@@ -1271,7 +1420,8 @@ qs_status run_ops(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm_un
                                (long long)(uintptr_t)s->d_rec, s->renorm_every,
                                s->xpass_impl * 16 + s->nbuf + 256 * s->tma_store + 1024 * s->xmerge +
                                    4096 * (int)s->tan_active + 8192 * s->pdl + 16384 * s->nbuf_shared +
-                                   65536 * s->shared_kernel + 131072 * s->c128_df + 262144 * (int)s->res_active,
+                                   65536 * s->shared_kernel + 131072 * s->c128_df + 262144 * (int)s->res_active +
+                                   524288 * (int)(s->plan_code != 0) + 1048576 * (int)s->shared_kernel_set,
                                s->method, (long long)s->dtype};
     if (!s->graph_exec || memcmp(key, s->graph_key, sizeof(key)) != 0) {
         if (s->graph_exec) { cudaGraphExecDestroy(s->graph_exec); s->graph_exec = nullptr; }
@@ -1519,6 +1669,21 @@ ScanParams scan12_params(const qs_sim *s, int n_points, int n_steps, int order, 
     return P;
 }
 
+// Shared-memory limits that no lattice changes, once per device.
+void set_fixed_attributes(int dev) {
+    static std::atomic<unsigned long long> done{0};
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done.load() & bit) return;
+    const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaFuncSetAttribute(k_energy<double>, A, (1 << LT) * 16);
+    cudaFuncSetAttribute(k_dos<float>, A, 64 * RED_THREADS * 8);
+    cudaFuncSetAttribute(k_dos<double>, A, 64 * RED_THREADS * 8);
+    cudaFuncSetAttribute(k_xpass_wide<W_GROUPS, 16>, A, 226 * 1024);
+    cudaFuncSetAttribute(k_xpass_wide<W_SLICE4, W_SLICE_WARPS>, A, 226 * 1024);
+    cudaFuncSetAttribute(k_xpass_wide<W_SLICE3, W_SLICE_WARPS>, A, 226 * 1024);
+    done.fetch_or(bit);
+}
+
 qs_status check_ready(qs_sim *s) {
     if (!s) return QS_ERR_ARG;
     if (!s->state[0]) FAIL(s, QS_ERR_STATE, "no state bound (qs_bind_state slot 0)");
@@ -1582,6 +1747,7 @@ qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch
     build_passes(s);
     build_variants(s);
     build_tma_passes(s);
+    build_wide_passes(s);
     auto fail = [&](const char *what) {
         g_create_error = what;
         qs_destroy(s);
@@ -1605,17 +1771,18 @@ qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch
     size_t pbytes = (size_t)RED_BLOCKS * batch * RED_NV * sizeof(double);
     size_t rbytes = (size_t)RES_SLOTS * batch * RED_NV * sizeof(double);
     if (cudaMalloc((void **)&s->d_partials, pbytes) != cudaSuccess) return fail("partials");
-    if (cudaMalloc((void **)&s->d_res, rbytes) != cudaSuccess) return fail("results");
-    if (cudaMemset(s->d_res, 0, rbytes) != cudaSuccess) return fail("results");
+    // results, and the error flag behind them
+    if (cudaMalloc((void **)&s->d_res, rbytes + sizeof(double)) != cudaSuccess) return fail("results");
+    if (cudaMemset(s->d_res, 0, rbytes + sizeof(double)) != cudaSuccess) return fail("results");
+    s->d_err = reinterpret_cast<int *>(s->d_res + (size_t)RES_SLOTS * batch * RED_NV);
     if (cudaMallocHost((void **)&s->h_res, rbytes + sizeof(double)) != cudaSuccess) return fail("pinned results");
     if (cudaEventCreateWithFlags(&s->rec_done, cudaEventDisableTiming) != cudaSuccess) return fail("event");
-    if (cudaMalloc((void **)&s->d_err, sizeof(int)) != cudaSuccess) return fail("error flag");
-    if (cudaMemset(s->d_err, 0, sizeof(int)) != cudaSuccess) return fail("error flag");
     {
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, dev);
         if (s->sm_count < 1) s->sm_count = 1;
+        set_fixed_attributes(dev);
         for (int nb = 2; nb <= 3; ++nb)
             for (int v = 0; v < 8; ++v)
                 cudaFuncSetAttribute(xpass_tma_kernel(nb, v & 1, (v >> 1) & 1, (v >> 2) & 1),
@@ -1639,9 +1806,6 @@ qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch
         cudaFuncSetAttribute(k_adj_xpass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
         cudaFuncSetAttribute(k_apply_h_pass<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
         cudaFuncSetAttribute(k_apply_h_pass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
-        cudaFuncSetAttribute(k_energy<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)((1 << LT) * 16));
-        cudaFuncSetAttribute(k_dos<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * RED_THREADS * 8);
-        cudaFuncSetAttribute(k_dos<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * RED_THREADS * 8);
         for (int v = 0; v < 3; ++v) {
             const bool tn = v >= 1, mg = v == 2;
             cudaFuncSetAttribute(adj_tma_kernel(2, tn, mg), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1668,7 +1832,6 @@ void qs_destroy(qs_sim *s) {
     cudaFree(s->d_rec);
     cudaFree(s->d_partials);
     cudaFree(s->d_res);
-    cudaFree(s->d_err);
     cudaFree(s->d_res_mail);
     cudaFree(s->d_adj_part);
     cudaFree(s->d_grad);
@@ -1745,7 +1908,7 @@ qs_status qs_set_option(qs_sim *s, int key, long long value) {
             s->c128_df = (int)value; return QS_OK;
         case QS_OPT_SHARED_KERNEL:
             if (value != 0 && value != 1) FAIL(s, QS_ERR_ARG, "shared-pass kernel must be 0 or 1");
-            s->shared_kernel = (int)value; return QS_OK;
+            s->shared_kernel = (int)value; s->shared_kernel_set = true; return QS_OK;
         case QS_OPT_ADJOINT:
             if (value < 0 || value > 7) FAIL(s, QS_ERR_ARG, "adjoint option must be 0..7");
             s->adj_impl = (value & 1) ? 1 : 0;
@@ -1774,8 +1937,8 @@ qs_status qs_set_option(qs_sim *s, int key, long long value) {
             if (value != 0 && sum != s->n - LT)
                 FAIL(s, QS_ERR_ARG, "the plan fuses %d new qubits, the state has %d beyond the first pass", sum,
                      s->n - LT);
+            s->plan_code = default_plan(s, k) ? 0 : value;   // (asked for by name, it is still the default)
             s->plan_k = k;
-            s->plan_code = value;
             return rebuild_plan(s);
         }
         default: FAIL(s, QS_ERR_ARG, "unknown option %d", key);
@@ -2284,7 +2447,7 @@ qs_status qs_autotune(qs_sim *s, int n_steps, int *best_xpass, int *best_buffers
         FAIL(s, QS_ERR_ARG, "null output");
     struct Cand { int xpass, nbuf, store, nsh, skern; };
     std::vector<Cand> cands;
-    if (s->passes.size() <= 2 && resident_fits(s))      // the default: resident, shared passes by form
+    if ((s->passes.size() <= 2 && resident_fits(s)) || !s->wide_maps.empty())   // the default
         cands.push_back({0, 3, 1, 0, 1});
     if (s->dtype == QS_C64 && s->tmaps_ok) {
         for (int nb = 2; nb <= 3; ++nb)
@@ -2376,6 +2539,7 @@ qs_status qs_autotune_plan(qs_sim *s, int n_steps, int *qubits_per_pass, int max
     size_t pick = 0;
     for (size_t i = 0; i < plans.size() && st == QS_OK; ++i) {
         s->plan_k = plans[i];
+        s->plan_code = default_plan(s, plans[i]) ? 0 : 1;
         if ((st = rebuild_plan(s)) != QS_OK) break;
         if ((st = qs_init_plus(s)) != QS_OK) break;
         if ((st = qs_evolve(s, c.data(), sv.data(), 0.02, 2, 2)) != QS_OK) break;   // warm-up
@@ -2400,7 +2564,8 @@ qs_status qs_autotune_plan(qs_sim *s, int n_steps, int *qubits_per_pass, int max
     }
     s->plan_k = plans[pick];
     s->plan_code = 0;
-    for (size_t j = 0; j < plans[pick].size(); ++j) s->plan_code |= (long long)plans[pick][j] << (4 * j);
+    for (size_t j = 0; j < plans[pick].size() && !default_plan(s, plans[pick]); ++j)
+        s->plan_code |= (long long)plans[pick][j] << (4 * j);
     if ((st = rebuild_plan(s)) != QS_OK) return st;
     *n_passes = qs_plan(s, qubits_per_pass, max);
     *best_ms_per_step = best / n_steps;

@@ -493,6 +493,8 @@ class Simulator:
             if self.n > 12:
                 self.set_option(QS_OPT_PLAN, plan_code(e["plan"]))
             self.set_option(QS_OPT_XPASS, e["xpass"])
+            if e["xpass"] == 0:                       # the default kernels
+                return e
             self.set_option(QS_OPT_TMA_BUFFERS, e["buffers"])
             self.set_option(QS_OPT_TMA_STORE, e["store"])
             self.set_option(QS_OPT_SHARED_BUFFERS, e["shared_buffers"])
