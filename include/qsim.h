@@ -86,10 +86,11 @@ typedef enum {
     QS_OPT_PROFILE = 2,       /* 1: time every fused X-pass launch with CUDA events on
                                  the bound stream (read with qs_profile_read)        */
     QS_OPT_GRAPH = 3,         /* 1: qs_evolve replays its launches as a CUDA graph    */
-    QS_OPT_XPASS = 4,         /* X-pass kernel: 0 auto: calls of twelve or more factor
-                                 groups on small states (up to 2^19 amplitudes in all;
-                                 any number of states of up to 12 qubits) run in one
-                                 launch with the state on the chip, others as 2; 1 the
+    QS_OPT_XPASS = 4,         /* X-pass kernel: 0 auto: small states (up to 2^19
+                                 amplitudes in all; any number of states of up to 12
+                                 qubits) run in one launch with the state on the chip
+                                 (beyond 12 qubits calls of up to 3 or at least 12
+                                 factor groups), others as 2; 1 the
                                  register-staged kernel, 2 the persistent TMA kernel
                                  (complex64; complex128: the double-float passes)    */
     QS_OPT_TMA_BUFFERS = 5,   /* shared-memory tile buffers per CTA of the TMA kernel:

@@ -412,9 +412,13 @@ namespace qsim {
 // triple once into shared memory (the triple per entry was a third of the FP64 work).
 // Blocks of 64 threads: FP64 issue bounds the kernel, so a short call spreads over SMs.
 constexpr int REC_THREADS = 64;
-__global__ void __launch_bounds__(REC_THREADS) k_build_records(RecGeom G, const DevCouplings *__restrict__ cpl,
-                                                               const double *__restrict__ sv, int op0,
+template <bool INLINE>
+__global__ void __launch_bounds__(REC_THREADS) k_build_records(RecGeom G, const double *__restrict__ in, size_t ncpl,
+                                                               const __grid_constant__ RecInline X, int op0,
                                                                double *__restrict__ recs) {
+    const double *src = INLINE ? X.v : in;
+    const DevCouplings *cpl = reinterpret_cast<const DevCouplings *>(src);
+    const double *sv = src + 4 * ncpl;
     const int nz = (G.nA + 1) * (G.nB + 1);
     const int nx = G.xlut_off > 0 ? (G.nXA + 1) * (G.nXB + 1) : 0;
     const int nt = G.tan_off > 0 ? nz : 0;

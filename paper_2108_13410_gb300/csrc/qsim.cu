@@ -148,6 +148,7 @@ struct qs_sim {
     // operator-record inputs (couplings, schedule) on the device
     double *d_in = nullptr; size_t d_in_cap = 0;
     bool in_path = false; size_t in_ncpl = 0;
+    bool in_inline = false; RecInline inl;     // short calls: in kernel parameters
     // scan workspaces
     double *d_scan = nullptr; size_t scan_cap = 0;
     int *d_queue = nullptr;                // work-queue counter of the mixed scan
@@ -1049,6 +1050,20 @@ qs_status upload_inputs(qs_sim *s, const qs_couplings *c, const double *sv, int 
     const int B = s->batch;
     const size_t ncpl = (size_t)B * (path ? n_steps : 1);
     const size_t in_doubles = ncpl * 4 + (path ? 0 : (size_t)n_steps);
+    auto fill = [&](double *dst) {
+        for (size_t i = 0; i < ncpl; ++i) {
+            dst[4 * i + 0] = c[i].J; dst[4 * i + 1] = c[i].h;
+            dst[4 * i + 2] = c[i].g; dst[4 * i + 3] = c[i].lambda;
+        }
+        if (!path) memcpy(dst + 4 * ncpl, sv, (size_t)n_steps * sizeof(double));
+    };
+    s->in_path = path;
+    s->in_ncpl = ncpl;
+    s->in_inline = in_doubles <= REC_INLINE;
+    if (s->in_inline) {
+        fill(s->inl.v);
+        return QS_OK;
+    }
     if (s->rec_pending) {
         CK(s, cudaEventSynchronize(s->rec_done));
         s->rec_pending = false;
@@ -1063,16 +1078,10 @@ qs_status upload_inputs(qs_sim *s, const qs_couplings *c, const double *sv, int 
     }
     qs_status st;
     if ((st = grow(s, &s->d_in, &s->d_in_cap, in_doubles, false)) != QS_OK) return st;
-    for (size_t i = 0; i < ncpl; ++i) {
-        s->h_rec[4 * i + 0] = c[i].J; s->h_rec[4 * i + 1] = c[i].h;
-        s->h_rec[4 * i + 2] = c[i].g; s->h_rec[4 * i + 3] = c[i].lambda;
-    }
-    if (!path) memcpy(s->h_rec + 4 * ncpl, sv, (size_t)n_steps * sizeof(double));
+    fill(s->h_rec);
     CK(s, cudaMemcpyAsync(s->d_in, s->h_rec, in_doubles * sizeof(double), cudaMemcpyHostToDevice, s->stream));
     CK(s, cudaEventRecord(s->rec_done, s->stream));
     s->rec_pending = true;
-    s->in_path = path;
-    s->in_ncpl = ncpl;
     return QS_OK;
 }
 
@@ -1104,8 +1113,8 @@ qs_status build_records(qs_sim *s, size_t op0, size_t n, double dt, int n_steps,
     const long long slices = (entries + REC_THREADS - 1) / REC_THREADS;
     const long long recs = (long long)n * B;
     const unsigned gy = (unsigned)std::max<long long>(1, std::min<long long>(slices, 8ll * s->sm_count / recs));
-    k_build_records<<<dim3((unsigned)recs, gy), REC_THREADS, 0, s->stream>>>(
-        G, reinterpret_cast<const DevCouplings *>(s->d_in), s->d_in + 4 * s->in_ncpl, (int)op0, s->d_rec);
+    auto kern = s->in_inline ? k_build_records<true> : k_build_records<false>;
+    kern<<<dim3((unsigned)recs, gy), REC_THREADS, 0, s->stream>>>(G, s->d_in, s->in_ncpl, s->inl, (int)op0, s->d_rec);
     CKL(s);
     s->launches++;
     return QS_OK;
@@ -1118,8 +1127,8 @@ qs_status build_call_records(qs_sim *s, size_t op0, size_t n, double dt, int n_s
     const ResParams &P = s->res;
     const size_t bytes = n * s->batch * (size_t)P.rec_bytes;
     if ((st = grow(s, &s->d_rec, &s->d_rec_cap, (bytes + 7) / 8, false)) != QS_OK) return st;
-    CK(s, resident_tables(P, record_geometry(s, dt, n_steps, order), reinterpret_cast<const DevCouplings *>(s->d_in),
-                          s->d_in + 4 * s->in_ncpl, (int)op0, (int)n, s->d_rec, s->sm_count, s->stream));
+    CK(s, resident_tables(P, record_geometry(s, dt, n_steps, order), s->d_in, s->in_ncpl, s->inl, s->in_inline, (int)op0,
+                          (int)n, s->d_rec, s->sm_count, s->stream));
     s->launches++;
     return QS_OK;
 }
@@ -1267,7 +1276,6 @@ bool df_schedule(const qs_sim *s) {
 // 13), 2^20 1.12 (20 qubits), 1.15 (4 x 18), 1.64 (16 x 16); double-float 2^18 0.48 (18 qubits),
 // 0.72 (4 x 16), 2^19 0.69 (19 qubits), 0.75 (4 x 17) but 1.4 (64 x 13), 2^20 1.24 (4 x 18);
 // FP64 2^18 0.37 to 0.51 (64 x 12).
-constexpr size_t RES_MIN_GROUPS = 12;
 
 bool resident_size(const qs_sim *s) {
     if (s->n < LT || (s->n == LT && s->dtype == QS_C64)) return true;
@@ -1313,14 +1321,16 @@ qs_status resident_mail(qs_sim *s) {
 }
 
 // A call runs resident by default (QS_OPT_XPASS auto, shared passes on, the default pass
-// plan, no per-pass profiling) from RES_MIN_GROUPS factor groups on, and with as many
-// between renormalisations: shorter runs keep one launch per pass, whose number
-// qs_launch_count reports to callers.
+// plan, no per-pass profiling).  Beyond one tile, runs of 4 to 11 factor groups keep one
+// launch per pass, whose number qs_launch_count reports to callers that rely on it; a single
+// step of 18 qubits (two groups, five launches there) takes 42 us in a loop, resident 26.
+bool resident_groups(const qs_sim *s, size_t groups) { return s->n <= LT || groups <= 3 || groups >= 12; }
+
 bool resident_call(qs_sim *s, size_t nops, int steps_per_renorm_unit) {
     if (s->method != 0 || s->xpass_impl != 0 || !s->xmerge || s->profile || s->passes.size() > 2) return false;
     if (s->dtype == QS_C128 && s->n > LT && !s->c128_df) return false;
-    if (nops < RES_MIN_GROUPS) return false;
-    if (s->renorm_every > 0 && (size_t)s->renorm_every * (size_t)std::max(1, steps_per_renorm_unit) < RES_MIN_GROUPS)
+    if (!resident_groups(s, nops)) return false;
+    if (s->renorm_every > 0 && !resident_groups(s, (size_t)s->renorm_every * (size_t)std::max(1, steps_per_renorm_unit)))
         return false;
     return resident_fits(s);
 }

@@ -24,6 +24,12 @@ struct RecGeom {
 
 struct DevCouplings { double J, h, g, lambda; };
 
+// The couplings and the schedule of a call that is short enough travel in the parameters of the
+// records kernel: no copy before it, and no wait of the host for the previous call's copy (which
+// held a loop over single steps at one call in flight).
+constexpr int REC_INLINE = 480;
+struct RecInline { double v[REC_INLINE]; };
+
 // The float pair within +-3 ulps of (u, s) that minimises |(1 - u)^2 + s^2 - m2|, the first
 // of equal ones by distance from (u, s).  With e0 the deviation of the rounded pair (FP64),
 // the deviation of a neighbour is e0 + du (du - 2 (1 - u0)) + ds (ds + 2 s0) with du, ds the

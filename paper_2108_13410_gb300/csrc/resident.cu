@@ -435,19 +435,26 @@ __global__ void __launch_bounds__((1 << (M - R)) + 32, min_ctas(M, R, sizeof(typ
     auto addr = [&](int set, long long l) -> long long {
         return !TWO || set == 0 ? (T << M) | l : (l & cm) | (T << P.c) | ((l >> P.c) << M);
     };
-    // table index of this thread's amplitudes in the layout of stage `st` of a set
+    // table index of this thread's amplitudes in the layout of stage `st` of a set: parity words
+    // of the thread's bits and of each register bit
     auto codes = [&](uint32_t (&code)[NRG / 2], int set, int st, const uint32_t *ca, const uint32_t *cb, int nb1) {
         const int b = st * R < M - R ? st * R : M - R;
+        const unsigned g0 = (unsigned)addr(set, W::pos(t, 0, b));
+        uint32_t wa[NRG], wb[NRG];
+        wa[0] = wb[0] = 0;
+        for (int q = 0; q < P.n; ++q)
+            if ((g0 >> q) & 1) { wa[0] ^= ca[q]; wb[0] ^= cb[q]; }
 #pragma unroll
-        for (int r = 0; r < NRG; ++r) {
-            const long long g = addr(set, W::pos(t, r, b));
-            uint32_t a = 0, bb = 0;
-            for (int q = 0; q < P.n; ++q)
-                if ((g >> q) & 1) { a ^= ca[q]; bb ^= cb[q]; }
-            const uint32_t idx = (uint32_t)(__popc(a) * nb1 + __popc(bb));
-            if (r & 1) code[r >> 1] |= idx << 16;
-            else code[r >> 1] = idx;
+        for (int k = 0; k < R; ++k) {
+            const int l = b + k, q = !TWO || set == 0 || l < P.c ? l : M + l - P.c;
+            const uint32_t xa = ca[q], xb = cb[q];       // (zero beyond the qubits)
+#pragma unroll
+            for (int r = 0; r < (1 << k); ++r) { wa[r | (1 << k)] = wa[r] ^ xa; wb[r | (1 << k)] = wb[r] ^ xb; }
         }
+#pragma unroll
+        for (int r = 0; r < NRG; r += 2)
+            code[r >> 1] = (uint32_t)(__popc(wa[r]) * nb1 + __popc(wb[r])) |
+                           (uint32_t)(__popc(wa[r + 1]) * nb1 + __popc(wb[r + 1])) << 16;
     };
     // Z tables: set 0 (two sets) or the layout that a round ends in; X tables (unitary gauge)
     // on set 1 or the low layout
@@ -613,11 +620,14 @@ __global__ void __launch_bounds__((1 << (M - R)) + 32, min_ctas(M, R, sizeof(typ
 // Operator records of the resident kernel: per factor group and state two tangents and the
 // group's cos factors C as a float (16 bytes each), the Z table (scaled by the group's cos factors in the tangent form) and the
 // Hadamard-basis X table, entries in the kernel's own format.  Geometry as k_build_records.
-template <class A>
-__global__ void __launch_bounds__(64) k_resident_tables(RecGeom G, const DevCouplings *__restrict__ cpl,
-                                                        const double *__restrict__ sv, int op0,
+template <class A, bool INLINE>
+__global__ void __launch_bounds__(64) k_resident_tables(RecGeom G, const double *__restrict__ in, size_t ncpl,
+                                                        const __grid_constant__ RecInline X, int op0,
                                                         unsigned char *__restrict__ recs,
                                                         const __grid_constant__ ResParams P) {
+    const double *src = INLINE ? X.v : in;
+    const DevCouplings *cpl = reinterpret_cast<const DevCouplings *>(src);
+    const double *sv = src + 4 * ncpl;
     const long long ob = blockIdx.x;
     const int op = op0 + (int)(ob / G.batch), b = (int)(ob % G.batch);
     __shared__ double tri[2][2];        // per X class: t, (1 + t^2)^n
@@ -772,17 +782,24 @@ cudaError_t resident_mail_clear(const ResParams &P, void *mail, cudaStream_t str
     return cudaGetLastError();
 }
 
-cudaError_t resident_tables(const ResParams &P, const RecGeom &G, const DevCouplings *cpl, const double *sv, int op0,
-                            int nops, void *recs, int sm_count, cudaStream_t stream) {
+template <class A>
+static void launch_tables(dim3 grid, cudaStream_t stream, const RecGeom &G, const double *in, size_t ncpl, const RecInline &X,
+                          bool inl, int op0, unsigned char *r, const ResParams &P) {
+    if (inl) k_resident_tables<A, true><<<grid, 64, 0, stream>>>(G, in, ncpl, X, op0, r, P);
+    else k_resident_tables<A, false><<<grid, 64, 0, stream>>>(G, in, ncpl, X, op0, r, P);
+}
+
+cudaError_t resident_tables(const ResParams &P, const RecGeom &G, const double *in, size_t ncpl, const RecInline &X,
+                            bool inl, int op0, int nops, void *recs, int sm_count, cudaStream_t stream) {
     const int entries = (P.nA + 1) * (P.nB + 1) + (P.had ? (P.nXA + 1) * (P.nXB + 1) : 0);
     const long long blocks = (long long)nops * G.batch;
     long long gy = (entries + 63) / 64, most = 8ll * sm_count / blocks;
     if (gy > most) gy = most < 1 ? 1 : most;
     const dim3 grid((unsigned)blocks, (unsigned)gy);
     unsigned char *r = (unsigned char *)recs;
-    if (P.arith == RES_F32) k_resident_tables<AF32><<<grid, 64, 0, stream>>>(G, cpl, sv, op0, r, P);
-    else if (P.arith == RES_DF) k_resident_tables<ADF><<<grid, 64, 0, stream>>>(G, cpl, sv, op0, r, P);
-    else k_resident_tables<AF64><<<grid, 64, 0, stream>>>(G, cpl, sv, op0, r, P);
+    if (P.arith == RES_F32) launch_tables<AF32>(grid, stream, G, in, ncpl, X, inl, op0, r, P);
+    else if (P.arith == RES_DF) launch_tables<ADF>(grid, stream, G, in, ncpl, X, inl, op0, r, P);
+    else launch_tables<AF64>(grid, stream, G, in, ncpl, X, inl, op0, r, P);
     return cudaGetLastError();
 }
 

@@ -37,8 +37,8 @@ bool resident_plan(ResParams &P, int arith, int n, int batch, int sm_count);
 size_t resident_mail_bytes(const ResParams &P);
 cudaError_t resident_mail_clear(const ResParams &P, void *mail, cudaStream_t stream);
 // Records of factor groups op0 .. op0 + nops - 1 (rec_bytes each, group-major).
-cudaError_t resident_tables(const ResParams &P, const RecGeom &G, const DevCouplings *cpl, const double *sv, int op0,
-                            int nops, void *recs, int sm_count, cudaStream_t stream);
+cudaError_t resident_tables(const ResParams &P, const RecGeom &G, const double *in, size_t ncpl, const RecInline &X,
+                            bool inl, int op0, int nops, void *recs, int sm_count, cudaStream_t stream);
 cudaError_t resident_launch(const ResParams &P, void *state, const void *recs, void *mail, int *err_flag,
                             cudaStream_t stream);
 constexpr int RES_MAX_GROUPS = 4096;
