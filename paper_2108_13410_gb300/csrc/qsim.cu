@@ -1127,7 +1127,9 @@ qs_status build_call_records(qs_sim *s, size_t op0, size_t n, double dt, int n_s
     const ResParams &P = s->res;
     const size_t bytes = n * s->batch * (size_t)P.rec_bytes;
     if ((st = grow(s, &s->d_rec, &s->d_rec_cap, (bytes + 7) / 8, false)) != QS_OK) return st;
-    CK(s, resident_tables(P, record_geometry(s, dt, n_steps, order), s->d_in, s->in_ncpl, s->inl, s->in_inline, (int)op0,
+    RecGeom G = record_geometry(s, dt, n_steps, order);
+    if (P.arith == RES_DF32) G.f32 = 0;
+    CK(s, resident_tables(P, G, s->d_in, s->in_ncpl, s->inl, s->in_inline, (int)op0,
                           (int)n, s->d_rec, s->sm_count, s->stream));
     s->launches++;
     return QS_OK;
@@ -1301,7 +1303,10 @@ bool resident_fits(qs_sim *s) {
             P.xcolB[q] = 1u << q;
             if (s->lat.x_class[q]) P.cls |= 1u << q;
         }
-        const int arith = s->dtype == QS_C64 ? RES_F32 : n <= LT ? RES_F64 : RES_DF;
+        // below 12 qubits the Walsh-Hadamard form in FP32 would round more than the per-factor
+        // kernels (a smooth state is one large amplitude in the Hadamard basis: energy error 1.3e-5
+        // against 4e-6 after 200 steps of 8 qubits), so complex64 states are carried in double-float
+        const int arith = s->dtype != QS_C64 ? (n <= LT ? RES_F64 : RES_DF) : P.had && n < LT ? RES_DF32 : RES_F32;
         if (resident_plan(P, arith, n, s->batch, s->sm_count)) s->res_known = 1;
     }
     return s->res_known == 1;

@@ -128,6 +128,16 @@ struct ADF {
     }
 };
 
+// complex64 states carried in double-float during the call
+struct ADF32 : ADF {
+    typedef float2 G;
+    static __device__ __forceinline__ V first(const G *g) { const float2 x = __ldcg(g); return V{pk(x.x, x.y), 0ull}; }
+    static __device__ __forceinline__ void last(G *g, const V &v) {
+        const float2 h = unpk(v.h), l = unpk(v.l);
+        __stcg(g, make_float2(h.x + l.x, h.y + l.y));
+    }
+};
+
 struct AF64 {
     static constexpr bool ROLLED = false, C_ALONE = false;
     typedef double2 V;
@@ -678,7 +688,7 @@ ResKernel pick32(bool had, bool two) {
 }
 
 size_t entry_bytes(int arith) {
-    return arith == RES_F32 ? sizeof(AF32::L) : arith == RES_DF ? sizeof(ADF::L) : sizeof(AF64::L);
+    return arith == RES_F32 ? sizeof(AF32::L) : arith == RES_F64 ? sizeof(AF64::L) : sizeof(ADF::L);
 }
 
 // complex64 and double-float: 16 amplitudes per thread; FP64: 2 per thread, since the FP64
@@ -692,6 +702,12 @@ ResKernel kernel_of(const ResParams &P, int *threads, size_t *smem, size_t tab_b
         return P.M == 7 ? pick<AF64, 7, 1>(P.had, P.two) : nullptr;
     }
     *threads = (int)(N >> 4) + 32;
+    if (P.arith == RES_DF32) {
+        *smem = 2 * N * 16 + lut;
+        if (P.two || !P.had) return nullptr;
+        return P.M == 9 ? k_resident<ADF32, 9, 4, true, false>
+                        : P.M == 10 ? k_resident<ADF32, 10, 4, true, false> : k_resident<ADF32, 11, 4, true, false>;
+    }
     if (P.arith == RES_DF) {
         *smem = 2 * N * 16 + lut;
         if (!P.two) return nullptr;
@@ -722,8 +738,8 @@ bool resident_plan(ResParams &P, int arith, int n, int batch, int sm_count) {
     P.n = n;
     int M, lo, hi;
     if (arith == RES_F64) { lo = hi = 7; }
-    else { lo = 9; hi = arith == RES_DF ? 11 : 12; }
-    const int one = arith == RES_F64 ? 7 : arith == RES_DF ? 0 : 12;   // largest single tile
+    else { lo = 9; hi = arith == RES_F32 ? 12 : 11; }
+    const int one = arith == RES_F64 ? 7 : arith == RES_DF ? 0 : arith == RES_DF32 ? 11 : 12;   // largest single tile
     P.two = n > one;
     if (!P.two) M = n < lo ? lo : n;
     else {
@@ -798,7 +814,7 @@ cudaError_t resident_tables(const ResParams &P, const RecGeom &G, const double *
     const dim3 grid((unsigned)blocks, (unsigned)gy);
     unsigned char *r = (unsigned char *)recs;
     if (P.arith == RES_F32) launch_tables<AF32>(grid, stream, G, in, ncpl, X, inl, op0, r, P);
-    else if (P.arith == RES_DF) launch_tables<ADF>(grid, stream, G, in, ncpl, X, inl, op0, r, P);
+    else if (P.arith != RES_F64) launch_tables<ADF>(grid, stream, G, in, ncpl, X, inl, op0, r, P);
     else launch_tables<AF64>(grid, stream, G, in, ncpl, X, inl, op0, r, P);
     return cudaGetLastError();
 }

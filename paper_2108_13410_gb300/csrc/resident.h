@@ -9,10 +9,10 @@ namespace qsim {
 
 constexpr int RES_MAXQ = 24;
 
-enum { RES_F32 = 0, RES_DF = 1, RES_F64 = 2 };   // arithmetic
+enum { RES_F32 = 0, RES_DF = 1, RES_F64 = 2, RES_DF32 = 3 };   // arithmetic
 
 struct ResParams {
-    int arith;                 // RES_F32 (complex64), RES_DF, RES_F64 (complex128)
+    int arith;                 // RES_F32, RES_DF32 (complex64), RES_DF, RES_F64 (complex128)
     int n, M;                  // qubits, tile bits
     int c;                     // two tile sets: chunk bits kept by the second one, 2 M - n
     int two;                   // 1: two tile sets with an exchange between them, 0: one tile per state
