@@ -157,8 +157,8 @@ typedef enum {
                                  the Walsh-Hadamard passes run in double-float
                                  arithmetic (each real number an unevaluated sum of two
                                  floats, 48 significand bits, on the FP32 pipes; the
-                                 state is converted in place to a blocked layout at the
-                                 start of a call and back at its end); 0: FP64
+                                 first pass of a call converts the state in place to a
+                                 blocked layout and the last one back); 0: FP64
                                  register-staged passes                               */
 } qs_option;
 

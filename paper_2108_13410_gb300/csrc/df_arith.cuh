@@ -140,4 +140,11 @@ __device__ __forceinline__ double float_to_double_bits(float f) {
     return __longlong_as_double((long long)d);
 }
 
+// (re, im) of a pair as complex128
+__device__ __forceinline__ double2 df_join(u64 vh, u64 vl) {
+    const float2 h = unpk(vh), l = unpk(vl);
+    return make_double2(float_to_double_bits(h.x) + float_to_double_bits(l.x),
+                        float_to_double_bits(h.y) + float_to_double_bits(l.y));
+}
+
 }  // namespace qsim

@@ -130,7 +130,9 @@ struct qs_sim {
     std::vector<CUtensorMap> tmaps_dfh, tmaps_dfl;
     bool tmaps_df_ok = false;
     int c128_df = 1;                       // QS_OPT_C128_DF
-    bool df_active = false;                // the state is in the blocked layout (inside a call)
+    bool df_active = false;                // inside a call with double-float passes
+    bool df_raw = false;                   // the state still holds complex128 (no pass launched yet)
+    struct { bool held = false, merged = false; int p = 0; const double *rec = nullptr, *rec2 = nullptr; TmaPass P; } df_last;
     bool tmaps_aux_ok = false;
     int *d_err = nullptr;                  // device flag: bounded wait gave up
     // adjoint workspaces
@@ -614,60 +616,6 @@ AdjKernel adj_tma_kernel(int nbuf, bool tan, bool merged = false, bool early = f
 }
 
 
-// One complex128 Walsh-Hadamard pass in double-float arithmetic over the blocked layout
-// (variants V_HAD, V_HAD_X, V_HAD_Z; merged: a second round of butterflies).
-size_t df_smem_bytes(const qs_sim *s) {
-    return 2 * (size_t)TMA_TILE_BYTES + 1024 + (size_t)s->max_lut * 32 + 3 * 256 * 8;
-}
-
-qs_status launch_xpass_df(qs_sim *s, int p, int variant, const double *rec, const double *rec2, int frame,
-                          int xscale) {
-    TmaPass P = s->tpasses[NVAR * p + variant];
-    const bool merged = rec2 != nullptr;
-    const bool rot = !P.hadamard;
-    P.frame = rot ? frame : 0;
-    P.xscale = rot ? xscale : 0;
-    if (rot && !(s->tan_active && (frame & 1)))
-        FAIL(s, QS_ERR_STATE, "double-float rotation passes run the tangent form only");
-    const size_t sm = df_smem_bytes(s);
-    auto kern = rot ? (merged ? k_xpass_df<true, true> : k_xpass_df<false, true>)
-                    : (merged ? k_xpass_df<true, false> : k_xpass_df<false, false>);
-    cudaEvent_t e1 = nullptr;
-    if (s->profile) {   // per-launch CUDA events, as for the complex64 passes
-        while (s->ev_pool.size() < s->ev_used + 2) {
-            cudaEvent_t e;
-            CK(s, cudaEventCreate(&e));
-            s->ev_pool.push_back(e);
-        }
-        cudaEvent_t e0 = s->ev_pool[s->ev_used];
-        e1 = s->ev_pool[s->ev_used + 1];
-        s->ev_used += 2;
-        s->ev_kind.resize(s->ev_used / 2);
-        s->ev_kind.back() = merged ? 1 : 0;
-        CK(s, cudaEventRecord(e0, s->stream));
-    }
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, sm);
-    if (per_sm < 1) per_sm = 1;
-    const long long g = std::min<long long>(P.total_tiles, (long long)per_sm * s->sm_count);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)g);
-    cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = s->stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = s->pdl ? 1 : 0;
-    CK(s, cudaLaunchKernelEx(&cfg, kern, (float2 *)s->state[0], rec, merged ? rec2 : rec, s->rec_stride, s->n - LT,
-                             s->d_err, s->tmaps_dfh[p], s->tmaps_dfl[p], P));
-    CKL(s);
-    s->launches++;
-    if (s->profile) CK(s, cudaEventRecord(e1, s->stream));
-    return QS_OK;
-}
-
 // CUDA events around a pass launch (QS_OPT_PROFILE): begin before it, *end recorded after it.
 qs_status profile_begin(qs_sim *s, bool merged, cudaEvent_t *end) {
     *end = nullptr;
@@ -717,17 +665,80 @@ qs_status launch_xpass_wide(qs_sim *s, int p, int variant, const double *rec, bo
     return QS_OK;
 }
 
-// In-place conversion of the bound complex128 state to (to_df) or from the blocked
-// double-float layout.
-qs_status df_convert(qs_sim *s, bool to_df) {
-    const long long amps = (long long)s->batch << s->n;
-    const unsigned grid = (unsigned)std::min<long long>((amps / 128 + 7) / 8, (long long)s->sm_count * 8);
-    if (to_df) k_df_split<<<grid, 256, 0, s->stream>>>((double2 *)s->state[0], amps);
-    else k_df_join<<<grid, 256, 0, s->stream>>>((double2 *)s->state[0], amps);
+size_t df_smem_bytes(const qs_sim *s) {
+    return 2 * (size_t)TMA_TILE_BYTES + 1024 + (size_t)s->max_lut * 32 + 3 * 256 * 8;
+}
+
+// Launch the pass that launch_xpass_df holds back; raw_out: the call's last one.
+qs_status df_launch_held(qs_sim *s, bool raw_out) {
+    if (!s->df_last.held) return QS_OK;
+    s->df_last.held = false;
+    TmaPass &P = s->df_last.P;
+    const bool merged = s->df_last.merged, rot = !P.hadamard;
+    const int p = s->df_last.p;
+    if (raw_out) P.raw |= 2;
+    const size_t sm = df_smem_bytes(s);
+    auto kern = rot ? (merged ? k_xpass_df<true, true> : k_xpass_df<false, true>)
+                    : (merged ? k_xpass_df<true, false> : k_xpass_df<false, false>);
+    cudaEvent_t end;
+    qs_status st = profile_begin(s, merged, &end);
+    if (st != QS_OK) return st;
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, sm);
+    if (per_sm < 1) per_sm = 1;
+    const long long g = std::min<long long>(P.total_tiles, (long long)per_sm * s->sm_count);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)g);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = s->pdl ? 1 : 0;
+    CK(s, cudaLaunchKernelEx(&cfg, kern, (float2 *)s->state[0], s->df_last.rec, s->df_last.rec2, s->rec_stride, s->n - LT,
+                             s->d_err, s->tmaps_dfh[p], s->tmaps_dfl[p], P));
     CKL(s);
     s->launches++;
-    s->df_active = to_df;
+    if (end) CK(s, cudaEventRecord(end, s->stream));
     return QS_OK;
+}
+
+// One pass in double-float arithmetic (variants V_HAD.. and V_ROT..; rec2: a second round).  It is
+// held back until the next one (or df_end) comes, so that the last pass of a call is known to
+// be the last: it writes complex128.
+qs_status launch_xpass_df(qs_sim *s, int p, int variant, const double *rec, const double *rec2, int frame,
+                          int xscale) {
+    TmaPass P = s->tpasses[NVAR * p + variant];
+    const bool rot = !P.hadamard;
+    P.frame = rot ? frame : 0;
+    P.xscale = rot ? xscale : 0;
+    if (rot && !(s->tan_active && (frame & 1)))
+        FAIL(s, QS_ERR_STATE, "double-float rotation passes run the tangent form only");
+    qs_status st = df_launch_held(s, false);
+    if (st != QS_OK) return st;
+    P.raw = s->df_raw ? 1 : 0;
+    s->df_raw = false;
+    s->df_last.held = true;
+    s->df_last.merged = rec2 != nullptr;
+    s->df_last.p = p;
+    s->df_last.rec = rec;
+    s->df_last.rec2 = rec2 ? rec2 : rec;
+    s->df_last.P = P;
+    return QS_OK;
+}
+
+// Begin and end of a run of double-float passes over the bound complex128 state.
+void df_begin(qs_sim *s) {
+    s->df_active = true;
+    s->df_raw = true;
+    s->df_last.held = false;
+}
+qs_status df_end(qs_sim *s) {
+    qs_status st = df_launch_held(s, true);
+    s->df_active = s->df_raw = false;
+    return st;
 }
 
 // One X pass.  rec2 != nullptr selects the merged TMA pass: X of the pass's qubits from
@@ -1014,10 +1025,11 @@ inline double res(const qs_sim *s, int slot, int b, int v) {
 template <typename R>
 qs_status renormalise(qs_sim *s) {
     qs_status st;
-    if (sizeof(R) == 8 && s->df_active) {   // blocked double-float layout: join, rescale, split
-        if ((st = df_convert(s, false)) != QS_OK) return st;
+    if (sizeof(R) == 8 && s->df_active) {   // double-float passes: back to complex128, rescale, go on
+        if ((st = df_end(s)) != QS_OK) return st;
         if ((st = renormalise<R>(s)) != QS_OK) return st;
-        return df_convert(s, true);
+        df_begin(s);
+        return QS_OK;
     }
     if ((st = reduce_diag<R>(s, s->state[0], 0, 0, false)) != QS_OK) return st;
     dim3 grid(152 * 8, (unsigned)s->batch);
@@ -1371,10 +1383,9 @@ qs_status launch_ops(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm
     if (s->res_active) return launch_ops_resident<R>(s, ops, steps_per_renorm_unit, j0, j1);
     if (merged_schedule<R>(s)) return launch_ops_merged<R>(s, ops, steps_per_renorm_unit, j0, j1);
     if (df_schedule<R>(s) && !s->df_active) {
-        // split into the blocked double-float layout, run the passes, join back
-        if ((st = df_convert(s, true)) != QS_OK) return st;
+        df_begin(s);
         st = launch_ops<R>(s, ops, steps_per_renorm_unit, j0, j1);
-        qs_status st2 = df_convert(s, false);
+        qs_status st2 = df_end(s);
         return st != QS_OK ? st : st2;
     }
     if (merged_schedule_ug<R>(s)) return launch_ops_merged_ug<R>(s, ops, steps_per_renorm_unit, j0, j1);

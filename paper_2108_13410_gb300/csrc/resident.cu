@@ -95,11 +95,7 @@ struct ADF {
         split_double(x.y, ih, il);
         return V{pk(rh, ih), pk(rl, il)};
     }
-    static __device__ __forceinline__ void last(G *g, const V &v) {
-        const float2 h = unpk(v.h), l = unpk(v.l);
-        __stcg(g, make_double2(float_to_double_bits(h.x) + float_to_double_bits(l.x),
-                               float_to_double_bits(h.y) + float_to_double_bits(l.y)));
-    }
+    static __device__ __forceinline__ void last(G *g, const V &v) { __stcg(g, df_join(v.h, v.l)); }
     static __device__ __forceinline__ T tan(double t) {
         const float a = __double2float_rn(t), b = __double2float_rn(t - (double)a);
         return T{pk(a, a), pk(b, b)};

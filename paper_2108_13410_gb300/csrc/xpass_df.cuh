@@ -18,7 +18,9 @@
 //     taken from it.)
 // Layout in HBM while a call runs ("blocked double-float"): every block of 16 amplitudes
 // (256 bytes of complex128) holds the 16 high (re, im) float pairs, then the 16 low pairs.
-// A block converts in place, and the high (low) halves of a tile form an ordinary
+// The first pass of a call splits the complex128 amplitudes of its tiles as it reads them and
+// the last one writes them back as complex128 (conversion kernels of their own took 2.1 of the
+// 24.4 ms of a five-step call at 27 qubits).  The high (low) halves of a tile form an ordinary
 // complex64-like tile under a tensor map with doubled strides (base, base + 128 bytes), so
 // the pass loads a tile pair by two TMA copies and reuses the stage layouts of the
 // complex64 kernel (xpass_tma.cuh).  The pass applies unnormalised Walsh-Hadamard
@@ -66,56 +68,6 @@ __device__ __forceinline__ void df_rotate(u64 (&h)[NR], u64 (&l)[NR], unsigned m
 #pragma unroll
         for (int r = 0; r < NR; ++r)
             if (!((r >> k) & 1)) df_rot_lazy(h[r], l[r], h[r | (1 << k)], l[r | (1 << k)], th, tl);
-    }
-}
-
-// In-place conversion of complex128 amplitudes to the blocked double-float layout and
-// back: a warp takes four runs of two 16-amplitude blocks (one amplitude per lane and
-// run, four loads in flight), reads them whole, and writes them after __syncwarp, so no
-// block is read after another lane wrote to it.  n_amps is a multiple of 128.
-constexpr int DF_RUNS = 4;
-
-__global__ void k_df_split(double2 *__restrict__ state, long long n_amps) {
-    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    const int lane = threadIdx.x & 31;
-    for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); 32 * DF_RUNS * w < n_amps;
-         w += warps) {
-        double2 v[DF_RUNS];
-#pragma unroll
-        for (int k = 0; k < DF_RUNS; ++k) v[k] = state[32 * (DF_RUNS * w + k) + lane];
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < DF_RUNS; ++k) {
-            const long long g = 32 * (DF_RUNS * w + k) + lane;
-            float rh, rl, ih, il;
-            split_double(v[k].x, rh, rl);
-            split_double(v[k].y, ih, il);
-            float2 *blk = reinterpret_cast<float2 *>(state + (g & ~15ll));
-            blk[g & 15] = make_float2(rh, ih);
-            blk[16 + (g & 15)] = make_float2(rl, il);
-        }
-    }
-}
-
-__global__ void k_df_join(double2 *__restrict__ state, long long n_amps) {
-    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    const int lane = threadIdx.x & 31;
-    for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); 32 * DF_RUNS * w < n_amps;
-         w += warps) {
-        float2 h[DF_RUNS], l[DF_RUNS];
-#pragma unroll
-        for (int k = 0; k < DF_RUNS; ++k) {
-            const long long g = 32 * (DF_RUNS * w + k) + lane;
-            const float2 *blk = reinterpret_cast<const float2 *>(state + (g & ~15ll));
-            h[k] = blk[g & 15];
-            l[k] = blk[16 + (g & 15)];
-        }
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < DF_RUNS; ++k)
-            state[32 * (DF_RUNS * w + k) + lane] =
-                make_double2(float_to_double_bits(h[k].x) + float_to_double_bits(l[k].x),
-                             float_to_double_bits(h[k].y) + float_to_double_bits(l[k].y));
     }
 }
 
@@ -251,8 +203,25 @@ __global__ void __launch_bounds__(NT, 2) k_xpass_df(float2 *__restrict__ state, 
         u64 *tl = reinterpret_cast<u64 *>(buf + (1 << LT));
         u64 h[NR], l[NR];
         // ---- stage A: registers = local 8..11 ----
+        if (P.raw & 1) {
+            // complex128 amplitudes under the two maps: a block's first eight in the high tile's
+            // row, the others in the low tile's; all are read before a half is written
+            const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(tlo & 8 ? tl : th);
+            const int unit = ((t >> 4) << 3) | ((tlo & 7) ^ ((t >> 4) & 7));
 #pragma unroll
-        for (int r = 0; r < NR; ++r) { h[r] = th[a_base + (r << TB)]; l[r] = tl[a_base + (r << TB)]; }
+            for (int r = 0; r < NR; ++r) {
+                const ulonglong2 x = src[unit + (r << 7)];
+                float rh, rl, ih, il;
+                split_double(__longlong_as_double((long long)x.x), rh, rl);
+                split_double(__longlong_as_double((long long)x.y), ih, il);
+                h[r] = pk(rh, ih);
+                l[r] = pk(rl, il);
+            }
+            __syncthreads();
+        } else {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) { h[r] = th[a_base + (r << TB)]; l[r] = tl[a_base + (r << TB)]; }
+        }
         const int pc_tile = __popcll(tile & tmask);
         if (ROT && (P.frame & 2)) {   // psi -> phi = i^popc psi
             const int k0 = __popc(t) + pc_tile;
@@ -361,13 +330,25 @@ __global__ void __launch_bounds__(NT, 2) k_xpass_df(float2 *__restrict__ state, 
             // blocked layout: amplitude g = 16 m + j has its high pair at float2 index
             // 32 m + j and its low pair at 32 m + 16 + j
             dst = reinterpret_cast<u64 *>(state) + 2 * (gbase + toff_a) + tlo;
+            if (P.raw & 2) {
+                double2 *o = reinterpret_cast<double2 *>(state) + gbase + toff_a + tlo;
 #pragma unroll
-            for (int r = 0; r < NR; ++r) { dst[2 * P.roff_a[r]] = h[r]; dst[2 * P.roff_a[r] + 16] = l[r]; }
+                for (int r = 0; r < NR; ++r) o[P.roff_a[r]] = df_join(h[r], l[r]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) { dst[2 * P.roff_a[r]] = h[r]; dst[2 * P.roff_a[r] + 16] = l[r]; }
+            }
         } else {
             df_renorm(h, l);
             dst = reinterpret_cast<u64 *>(state) + 2 * (gbase + toff_c) + tlo;
+            if (P.raw & 2) {
+                double2 *o = reinterpret_cast<double2 *>(state) + gbase + toff_c + tlo;
 #pragma unroll
-            for (int r = 0; r < NR; ++r) { dst[2 * P.roff_c[r]] = h[r]; dst[2 * P.roff_c[r] + 16] = l[r]; }
+                for (int r = 0; r < NR; ++r) o[P.roff_c[r]] = df_join(h[r], l[r]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) { dst[2 * P.roff_c[r]] = h[r]; dst[2 * P.roff_c[r] + 16] = l[r]; }
+            }
         }
     }
 }
