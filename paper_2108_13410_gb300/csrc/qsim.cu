@@ -1545,11 +1545,16 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
         Gt = (unsigned)std::min<long long>((long long)B << (s->n - LT), (long long)per_sm * s->sm_count);
     }
     const size_t nblk_t = (size_t)np * Gt;
-    // TMA path: one partial-sum region per factor group, two used in turn (a shared reverse
-    // pass writes the terms of two consecutive groups)
+    // TMA path: one partial-sum region per factor group, in two rings of F regions (8 MB) used in
+    // turn, so that one memset clears and one launch sums F groups (one of each per group took
+    // 8 of 29 us a group at 18 qubits).  A shared reverse pass also writes the terms of the next
+    // lower group, which may lie in the other ring: it is cleared a ring ahead.
     const size_t region = nblk_t * B * RED_NV;
-    if ((st = grow(s, &s->d_adj_part, &s->adj_part_cap, std::max(nblk * B * RED_NV, 2 * region), false)) != QS_OK)
+    const size_t F = std::max<size_t>(1, std::min<size_t>(nops, (8u << 20) / (region * sizeof(double))));
+    const size_t ring = F * region;
+    if ((st = grow(s, &s->d_adj_part, &s->adj_part_cap, std::max(nblk * B * RED_NV, 2 * ring), false)) != QS_OK)
         return st;
+    auto region_of = [&](size_t op) { return s->d_adj_part + ((op / F) & 1) * ring + (op % F) * region; };
     // shared reverse passes: consecutive factor groups meet on one qubit group, as in the
     // forward sweep (orders ga, 0 .. np-3, gb and gb, 0 .. np-3, ga; ga = np-2, gb = np-1)
     const bool share = adj_tan && s->xmerge && np >= 2;
@@ -1574,8 +1579,11 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
         }
         const double *rec = s->d_rec + (jj - chunk0) * B * (size_t)s->rec_stride;
         if (use_tma) {
-            double *part_j = s->d_adj_part + (jj & 1) * region;
-            if (!carried) CK(s, cudaMemsetAsync(part_j, 0, region * sizeof(double), s->stream));
+            double *part_j = region_of(jj);
+            if (jj + 1 == nops)
+                CK(s, cudaMemsetAsync(s->d_adj_part + ((jj / F) & 1) * ring, 0, ring * sizeof(double), s->stream));
+            if ((jj + 1 == nops || jj % F == F - 1) && jj >= F)
+                CK(s, cudaMemsetAsync(s->d_adj_part + ((jj / F - 1) & 1) * ring, 0, ring * sizeof(double), s->stream));
             // X qubits per class already un-rotated in this factor group
             int done[2] = {carried ? carry_done[0] : 0, carried ? carry_done[1] : 0};
             bool next_carried = false;
@@ -1595,9 +1603,8 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
                 const bool merge = share && last && jj >= 1 && jj - 1 >= chunk0 && ops[(jj - 1) * B].has_z;
                 if (merge) {
                     // last pass of op jj, Z layer and first pass of op jj-1 on the same qubits
-                    double *part_prev = s->d_adj_part + ((jj - 1) & 1) * region;
+                    double *part_prev = region_of(jj - 1);
                     const double *rec_prev = rec - B * (size_t)s->rec_stride;
-                    CK(s, cudaMemsetAsync(part_prev, 0, region * sizeof(double), s->stream));
                     int d2[2] = {0, 0};
                     for (int stg = 2; stg >= 0; --stg) {     // second rotation round runs C, B, A
                         P.adj_u2[stg][0] = s->nX0 - d2[0];
@@ -1635,8 +1642,12 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
             }
             if (done[0] != s->nX0 || done[1] != s->nX1)
                 FAIL(s, QS_ERR_STATE, "reverse passes do not cover every X qubit once");
-            k_finish<RED_NV><<<B, RED_THREADS, 0, s->stream>>>(part_j, (int)nblk_t, 4, s->d_grad + jj * B * RED_NV);
-            CKL(s); s->launches++;
+            if (jj % F == 0) {      // every term of this ring's groups is in
+                const size_t cnt = std::min(F, nops - jj);
+                k_finish<RED_NV><<<(unsigned)(cnt * B), RED_THREADS, 0, s->stream>>>(part_j, (int)nblk_t, 4,
+                                                                                     s->d_grad + jj * B * RED_NV);
+                CKL(s); s->launches++;
+            }
             carried = next_carried;
             continue;
         }
