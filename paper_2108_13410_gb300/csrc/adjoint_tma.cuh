@@ -183,6 +183,9 @@ __global__ void __launch_bounds__(NT, NBUF == 1 ? 2 : 1) k_adj_tma(float2 *__res
         ptab[e] = make_uint2(a, b);
     }
     __syncthreads();
+    // the set-up above may overlap the previous kernel; reads of global memory may not
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     auto issue = [&](int it) {
         long long tile = first + (long long)it * G;
@@ -307,7 +310,7 @@ __global__ void __launch_bounds__(NT, NBUF == 1 ? 2 : 1) k_adj_tma(float2 *__res
                         const double q0 = 1.0 + rr[P.tan_off] * rr[P.tan_off];
                         const double q1 = 1.0 + rr[P.tan_off + 1] * rr[P.tan_off + 1];
                         const int *u = round ? P.adj_u2[st] : P.adj_u[st];
-                        s_corr[round][st] = (float)(pow(q0, (double)u[0]) * pow(q1, (double)u[1]));
+                        s_corr[round][st] = (float)(dev_powi(q0, u[0]) * dev_powi(q1, u[1]));
                     }
                 }
             }

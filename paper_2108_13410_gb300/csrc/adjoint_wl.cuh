@@ -72,6 +72,9 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_adj_wl(float2 *__restrict__ p
         ptab[e] = make_uint2(a, b);
     }
     for (int e = t; e < NW * 8; e += NTH) red[e / 8][e % 8] = 0.0;
+    // the set-up above may overlap the previous kernel; reads of global memory may not
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // records of the single batch element: round 0 this factor group (stages A, C),
     // round 1 the previous one (stages C, A); inverse factor a' = a - t b, b' = b + t a
     if (t < 2 * 3 * RB) {
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_adj_wl(float2 *__restrict__ p
             const double q0 = 1.0 + rr[P.tan_off] * rr[P.tan_off];
             const double q1 = 1.0 + rr[P.tan_off + 1] * rr[P.tan_off + 1];
             const int *u = round ? P.adj_u2[st] : P.adj_u[st];
-            s_corr[round][st] = (float)(pow(q0, (double)u[0]) * pow(q1, (double)u[1]));
+            s_corr[round][st] = (float)(dev_powi(q0, u[0]) * dev_powi(q1, u[1]));
         }
     }
     const int nB1 = P.nB + 1, nlut = (P.nA + 1) * nB1;

@@ -1545,12 +1545,12 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
         Gt = (unsigned)std::min<long long>((long long)B << (s->n - LT), (long long)per_sm * s->sm_count);
     }
     const size_t nblk_t = (size_t)np * Gt;
-    // TMA path: one partial-sum region per factor group, in two rings of F regions (8 MB) used in
+    // TMA path: one partial-sum region per factor group, in two rings of F regions (512 KB) used in
     // turn, so that one memset clears and one launch sums F groups (one of each per group took
     // 8 of 29 us a group at 18 qubits).  A shared reverse pass also writes the terms of the next
     // lower group, which may lie in the other ring: it is cleared a ring ahead.
     const size_t region = nblk_t * B * RED_NV;
-    const size_t F = std::max<size_t>(1, std::min<size_t>(nops, (8u << 20) / (region * sizeof(double))));
+    const size_t F = std::max<size_t>(1, std::min<size_t>(nops, (1u << 19) / (region * sizeof(double))));
     const size_t ring = F * region;
     if ((st = grow(s, &s->d_adj_part, &s->adj_part_cap, std::max(nblk * B * RED_NV, 2 * ring), false)) != QS_OK)
         return st;
@@ -1564,6 +1564,23 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
         ord[0][i] = i == 0 ? np - 2 : (i == np - 1 ? np - 1 : i - 1);
         ord[1][i] = i == 0 ? np - 1 : (i == np - 1 ? np - 2 : i - 1);
     }
+    // reverse passes: programmatic stream serialisation, as the forward ones
+    auto launch = [&](auto kern, unsigned grid, int threads, size_t smem_bytes, const double *rec, double *part, int slot0,
+                      int zinv, const double *rec2, double *part2, int p, const TmaPass &P) -> qs_status {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem_bytes;
+        cfg.stream = s->stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = s->pdl ? 1 : 0;
+        CK(s, cudaLaunchKernelEx(&cfg, kern, (float2 *)s->state[0], (float2 *)s->state[1], rec, s->rec_stride, s->n - LT,
+                                 s->d_err, part, (int)nblk_t, slot0, zinv, rec2, part2, 0, s->tmaps[p], s->tmaps_aux[p], P));
+        return QS_OK;
+    };
     bool carried = false;   // the first qubit group of op jj was un-rotated by op jj+1's last pass
     int dir = 0, carry_done[2] = {0, 0};
     if ((st = grow(s, &s->d_grad, &s->grad_cap, nops * B * RED_NV, false)) != QS_OK) return st;
@@ -1621,23 +1638,17 @@ qs_status adjoint_impl(qs_sim *s, const qs_couplings *c, const double *sv, doubl
                         // it (measured against 10, 11, 14 and 16 warps and the later reload)
                         const size_t wsm = 2 * (size_t)TMA_TILE_BYTES * 3 + 1024 + (size_t)s->max_lut * 8 + 3 * 256 * 8;
                         const unsigned gw = (unsigned)std::min<long long>(P.total_tiles, (long long)s->sm_count);
-                        k_adj_wl<3, 12, 1, 0><<<gw, 384, wsm, s->stream>>>(
-                            (float2 *)s->state[0], (float2 *)s->state[1], rec, s->rec_stride, s->n - LT, s->d_err,
-                            part_j, (int)nblk_t, i * (int)Gt, 0, rec_prev, part_prev, 0, s->tmaps[p], s->tmaps_aux[p],
-                            P);
+                        st = launch(k_adj_wl<3, 12, 1, 0>, gw, 384, wsm, rec, part_j, i * (int)Gt, 0, rec_prev, part_prev, p, P);
                     } else {
-                        adj_kern_m<<<Gt, adj_threads, adj_smem, s->stream>>>(
-                            (float2 *)s->state[0], (float2 *)s->state[1], rec, s->rec_stride, s->n - LT, s->d_err,
-                            part_j, (int)nblk_t, i * (int)Gt, 0, rec_prev, part_prev, 0, s->tmaps[p], s->tmaps_aux[p],
-                            P);
+                        st = launch(adj_kern_m, Gt, adj_threads, adj_smem, rec, part_j, i * (int)Gt, 0, rec_prev, part_prev, p,
+                                    P);
                     }
                     next_carried = true;
                     dir ^= 1;
                 } else {
-                    adj_kern<<<Gt, adj_threads, adj_smem, s->stream>>>(
-                        (float2 *)s->state[0], (float2 *)s->state[1], rec, s->rec_stride, s->n - LT, s->d_err, part_j,
-                        (int)nblk_t, i * (int)Gt, zinv, rec, part_j, 0, s->tmaps[p], s->tmaps_aux[p], P);
+                    st = launch(adj_kern, Gt, adj_threads, adj_smem, rec, part_j, i * (int)Gt, zinv, rec, part_j, p, P);
                 }
+                if (st != QS_OK) return st;
                 CKL(s); s->launches++;
             }
             if (done[0] != s->nX0 || done[1] != s->nX1)

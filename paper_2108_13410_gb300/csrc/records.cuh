@@ -180,4 +180,12 @@ __device__ inline void dev_scaled_pair(bool f32, double phi, double C, double *o
     dev_nearest_modulus((1.0 - C) + C * 2.0 * sh * sh, C * 2.0 * sh * ch, C * C, ou, os);
 }
 
+// x^n by squaring (pow costs a small pass microseconds of FP64 latency)
+__device__ inline double dev_powi(double x, int n) {
+    double p = 1.0;
+    for (; n; n >>= 1, x *= x)
+        if (n & 1) p *= x;
+    return p;
+}
+
 }  // namespace qsim
