@@ -181,6 +181,21 @@ def qs_init_toric(sim, which: int):
     _check(sim, library().qs_init_toric(sim, which))
 
 
+def _path_records(flat):
+    """Records (g, lambda, J, h) of plain numbers as one array in the layout of qs_couplings, or
+    None for anything else (shorter records, dicts, qs_couplings), which _couplings takes record
+    by record at 1 us each."""
+    if not flat or not isinstance(flat[0], tuple) or len(flat[0]) != 4:
+        return None
+    try:
+        a = np.array(flat)
+    except ValueError:                       # records of different lengths
+        return None
+    if a.ndim != 2 or a.shape[1] != 4 or a.dtype.kind not in "fiu":
+        return None
+    return np.ascontiguousarray(a.astype(np.float64, copy=False)[:, [2, 3, 0, 1]])
+
+
 def qs_evolve_path(sim, per_step, dt: float, order: int, batch: int = 1):
     """per_step: sequence of n_steps coupling records (batch 1) or of n_steps lists of
     `batch` records; step k evolves under H1 with those couplings.  A float64 numpy array
@@ -203,7 +218,8 @@ def qs_evolve_path(sim, per_step, dt: float, order: int, batch: int = 1):
             assert len(rec) == batch
             flat.extend(rec)
     n_steps = len(flat) // batch
-    arr = _couplings(flat, len(flat))
+    rec = _path_records(flat)
+    arr = _couplings(flat, len(flat)) if rec is None else rec.ctypes.data_as(ctypes.POINTER(qs_couplings))
     _check(sim, library().qs_evolve_path(sim, arr, dt, n_steps, order))
 
 
@@ -493,12 +509,11 @@ class Simulator:
             if self.n > 12:
                 self.set_option(QS_OPT_PLAN, plan_code(e["plan"]))
             self.set_option(QS_OPT_XPASS, e["xpass"])
-            if e["xpass"] == 0:                       # the default kernels
-                return e
             self.set_option(QS_OPT_TMA_BUFFERS, e["buffers"])
             self.set_option(QS_OPT_TMA_STORE, e["store"])
             self.set_option(QS_OPT_SHARED_BUFFERS, e["shared_buffers"])
-            self.set_option(QS_OPT_SHARED_KERNEL, e["shared_kernel"])
+            if e["xpass"] != 0:                       # 0: the default kernels, none set by name
+                self.set_option(QS_OPT_SHARED_KERNEL, e["shared_kernel"])
             return e
         plan, plan_ms = (qs_autotune_plan(self.h, n_steps) if self.n > 12 else (qs_plan(self.h), None))
         xp, nb, so, ns, sk, ms = qs_autotune(self.h, n_steps)
