@@ -189,7 +189,8 @@ def _path_records(flat):
         return None
     try:
         a = np.array(flat)
-    except ValueError:                       # records of different lengths
+    except (ValueError, TypeError, RuntimeError):   # other lengths; numbers numpy cannot take, e.g.
+                                                    # scalars on a device or with gradients
         return None
     if a.ndim != 2 or a.shape[1] != 4 or a.dtype.kind not in "fiu":
         return None

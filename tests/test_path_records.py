@@ -17,6 +17,26 @@ def test_same_bytes(flat):
     assert a.tobytes() == ctypes.string_at(ctypes.addressof(b), ctypes.sizeof(b))
 
 
+class _Scalar:
+    """A number that converts by float() only, as a tensor on a device does."""
+
+    def __init__(self, error):
+        self.error = error
+
+    def __float__(self):
+        return 0.5
+
+    def __array__(self, *args, **kwargs):
+        raise self.error("not an array")
+
+
+@pytest.mark.parametrize("error", [TypeError, RuntimeError, ValueError])
+def test_numbers_numpy_refuses_are_left_alone(error):
+    flat = [(_Scalar(error), 0.2, 0.5, 0.7)]
+    assert Q._path_records(flat) is None
+    assert Q._couplings(flat, 1)[0].g == 0.5
+
+
 @pytest.mark.parametrize("flat", [
     [], [(0.1, 0.2)], [(0.1, 0.2, 0.5)], [(0.1, 0.2, 0.5, 0.7), (0.1, 0.2)], [{"g": 0.1, "lambda": 0.2}],
     [[0.1, 0.2, 0.5, 0.7]], [(0.1, 0.2, "0.5", 0.7)], [(0.1, 0.2, None, 0.7)], [(0.1, 0.2, 1j, 0.7)],
