@@ -1414,6 +1414,11 @@ qs_status run_ops(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm_un
     // away from 1, where rounding u would cost relative precision in C
     s->tan_active = false;
     s->res_active = resident_call(s, nops, steps_per_renorm_unit);
+    // no memory for the mail boxes: the passes, which need none
+    if (s->res_active && (st = resident_mail(s)) != QS_OK) {
+        if (st != QS_ERR_OOM) return st;
+        s->res_active = false;
+    }
     const bool tma_path = sizeof(R) == 4 ? s->tmaps_ok : (s->c128_df && s->tmaps_df_ok);
     if (s->method == 0 && s->lat.gauge_higgs && (tma_path || s->res_active) && s->xpass_impl != 1) {
         bool ok = true;
@@ -1426,7 +1431,6 @@ qs_status run_ops(qs_sim *s, const std::vector<Op> &ops, int steps_per_renorm_un
         s->res_active = s->res_active && ok;
     }
     if (s->method == 0) {
-        if (s->res_active && (st = resident_mail(s)) != QS_OK) return st;
         if ((st = upload_inputs(s, c, sv, n_steps, path)) != QS_OK) return st;
         if (nops > REC_CHUNK) {
             // long schedules: records of REC_CHUNK ops at a time, direct launches
