@@ -29,8 +29,9 @@
 // Tables and rotation constants of the next pass are copied from the operator records while a
 // pass runs, and the table index of each amplitude (a CTA's tiles do not change) is computed
 // once per launch.
-// Waits are bounded (about a second), after which the error flag is set and every CTA
-// leaves; the launch is cooperative, so all CTAs of a state are resident.
+// The polls of the mail boxes are bounded (about a second), after which the error flag is set and
+// every CTA leaves; the launch is cooperative, so all CTAs of a state are resident.  The named
+// barriers inside a CTA have no limit: every warp reaches each of them.
 #include "resident.h"
 
 #include "df_arith.cuh"
@@ -219,6 +220,19 @@ __device__ __forceinline__ void copy_async16(void *dst, const void *src) {
 __device__ __forceinline__ void copy_async_wait() {
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
+// Named barriers of a CTA.  They take converged warps (aligned forms: a split warp would count
+// early, or twice), so lanes that may be apart, after a lane's fence, a copy loop or a poll that
+// some lanes leave earlier, meet first.  The workers' own barrier (1) comes after straight-line
+// code, except behind the poll, where receive() joins the warp.
+template <int ID, int N> __device__ __forceinline__ void barrier_sync() {
+    if (ID != 1) __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory");
+}
+template <int ID, int N> __device__ __forceinline__ void barrier_arrive() {
+    if (ID != 1) __syncwarp();
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(N) : "memory");
+}
+
 // slot of tile amplitude l: the low four bits xor bits 4..7, so that 16 (8) consecutive
 // lanes of every stage layout hit different 8-byte (16-byte) bank groups
 __device__ __forceinline__ int slot(int l) { return l ^ ((l >> 4) & 15); }
@@ -261,7 +275,7 @@ struct Worker {
     static __device__ __forceinline__ int pos(int t, int r, int b) {
         return (t & ((1 << b) - 1)) | (r << b) | ((t >> b) << (b + R));
     }
-    __device__ __forceinline__ void sync() { asm volatile("bar.sync 1, %0;" ::"n"(NTH) : "memory"); }
+    __device__ __forceinline__ void sync() { barrier_sync<1, NTH>(); }
     // registers from the layout of stage SF to that of stage ST
     template <int SF, int ST> __device__ __forceinline__ void move() {
         S *p = tile + buf * N;
@@ -390,10 +404,10 @@ __global__ void __launch_bounds__((1 << (M - R)) + 32, min_ctas(M, R, sizeof(typ
     const int grp = TWO ? (int)blockIdx.x / P.tiles : (int)blockIdx.x;
     const long long T = TWO ? (int)blockIdx.x % P.tiles : 0;
     const int n_pass = HAD ? 2 * P.nops : P.nops;
-    auto received = [&]() { asm volatile("bar.arrive 2, %0;" ::"n"(NTH + 32) : "memory"); };
-    auto may_send = [&]() { asm volatile("bar.sync 3, %0;" ::"n"(NTH + 32) : "memory"); };
+    auto received = [&]() { barrier_arrive<2, NTH + 32>(); };
+    auto may_send = [&]() { barrier_sync<3, NTH + 32>(); };
     // end of a state: the tables are free and every barrier-3 phase is over
-    auto state_done = [&]() { asm volatile("bar.sync 2, %0;" ::"n"(NTH + 32) : "memory"); };
+    auto state_done = [&]() { barrier_sync<2, NTH + 32>(); };
     if (t == 0) s_ok = 1;
     __syncthreads();
     if (t >= NTH) {
@@ -403,7 +417,7 @@ __global__ void __launch_bounds__((1 << (M - R)) + 32, min_ctas(M, R, sizeof(typ
             auto rec_of = [&](int op) { return recs + ((long long)op * P.batch + b) * P.rec_bytes; };
             for (int k = -1; k < n_pass; ++k) {
                 if (k >= 0) {
-                    asm volatile("bar.sync 2, %0;" ::"n"(NTH + 32) : "memory");
+                    barrier_sync<2, NTH + 32>();
                     if (!*(volatile int *)&s_ok) return;
                 }
                 if (k + 1 < n_pass) {                          // the table of pass k + 1
@@ -421,7 +435,7 @@ __global__ void __launch_bounds__((1 << (M - R)) + 32, min_ctas(M, R, sizeof(typ
                 }
                 if (TWO && lane == 0 && k >= 0) __threadfence();
                 copy_async_wait();
-                asm volatile("bar.arrive 3, %0;" ::"n"(NTH + 32) : "memory");
+                barrier_arrive<3, NTH + 32>();
             }
             state_done();
         }
@@ -578,6 +592,7 @@ __global__ void __launch_bounds__((1 << (M - R)) + 32, min_ctas(M, R, sizeof(typ
             }
 #pragma unroll
             for (int r = 0; r < NRG; ++r) { clear(p + off_of(set, r)); w.v[r] = A::from(x[r]); }
+            __syncwarp();
             w.sync();
             received();
             return *(volatile int *)&s_ok != 0;
