@@ -132,7 +132,7 @@ struct qs_sim {
     int c128_df = 1;                       // QS_OPT_C128_DF
     bool df_active = false;                // inside a call with double-float passes
     bool df_raw = false;                   // the state still holds complex128 (no pass launched yet)
-    struct { bool held = false, merged = false; int p = 0; const double *rec = nullptr, *rec2 = nullptr; TmaPass P; } df_last;
+    struct { bool held = false, merged = false; int p = 0, raw = 0; const double *rec = nullptr, *rec2 = nullptr; TmaPass P; } df_last;
     bool tmaps_aux_ok = false;
     int *d_err = nullptr;                  // device flag: bounded wait gave up
     // adjoint workspaces
@@ -669,6 +669,19 @@ size_t df_smem_bytes(const qs_sim *s) {
     return 2 * (size_t)TMA_TILE_BYTES + 1024 + (size_t)s->max_lut * 32 + 3 * 256 * 8;
 }
 
+typedef void (*DfKernel)(float2 *, const double *, const double *, int, int, int *, CUtensorMap, CUtensorMap, TmaPass);
+
+template <int RAW>
+DfKernel df_kernel_raw(bool merged, bool rot) {
+    return rot ? (merged ? k_xpass_df<true, true, RAW> : k_xpass_df<false, true, RAW>)
+               : (merged ? k_xpass_df<true, false, RAW> : k_xpass_df<false, false, RAW>);
+}
+
+DfKernel df_kernel(bool merged, bool rot, int raw) {
+    return raw == 0 ? df_kernel_raw<0>(merged, rot) : raw == 1 ? df_kernel_raw<1>(merged, rot)
+         : raw == 2 ? df_kernel_raw<2>(merged, rot) : df_kernel_raw<3>(merged, rot);
+}
+
 // Launch the pass that launch_xpass_df holds back; raw_out: the call's last one.
 qs_status df_launch_held(qs_sim *s, bool raw_out) {
     if (!s->df_last.held) return QS_OK;
@@ -676,10 +689,8 @@ qs_status df_launch_held(qs_sim *s, bool raw_out) {
     TmaPass &P = s->df_last.P;
     const bool merged = s->df_last.merged, rot = !P.hadamard;
     const int p = s->df_last.p;
-    if (raw_out) P.raw |= 2;
     const size_t sm = df_smem_bytes(s);
-    auto kern = rot ? (merged ? k_xpass_df<true, true> : k_xpass_df<false, true>)
-                    : (merged ? k_xpass_df<true, false> : k_xpass_df<false, false>);
+    const DfKernel kern = df_kernel(merged, rot, s->df_last.raw | (raw_out ? 2 : 0));
     cudaEvent_t end;
     qs_status st = profile_begin(s, merged, &end);
     if (st != QS_OK) return st;
@@ -718,7 +729,7 @@ qs_status launch_xpass_df(qs_sim *s, int p, int variant, const double *rec, cons
         FAIL(s, QS_ERR_STATE, "double-float rotation passes run the tangent form only");
     qs_status st = df_launch_held(s, false);
     if (st != QS_OK) return st;
-    P.raw = s->df_raw ? 1 : 0;
+    s->df_last.raw = s->df_raw ? 1 : 0;
     s->df_raw = false;
     s->df_last.held = true;
     s->df_last.merged = rec2 != nullptr;
@@ -1839,10 +1850,9 @@ qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch
             for (int v = 0; v < 8; ++v)
                 cudaFuncSetAttribute(xpass_tma_kernel(nb, v & 1, (v >> 1) & 1, (v >> 2) & 1),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tma_smem_bytes(s, nb, true));
-        cudaFuncSetAttribute(k_xpass_df<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)df_smem_bytes(s));
-        cudaFuncSetAttribute(k_xpass_df<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)df_smem_bytes(s));
-        cudaFuncSetAttribute(k_xpass_df<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)df_smem_bytes(s));
-        cudaFuncSetAttribute(k_xpass_df<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)df_smem_bytes(s));
+        for (int v = 0; v < 16; ++v)
+            cudaFuncSetAttribute(df_kernel(v & 1, (v >> 1) & 1, v >> 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)df_smem_bytes(s));
         cudaFuncSetAttribute(k_adj_wl<3, 12, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(2 * (size_t)TMA_TILE_BYTES * 3 + 1024 + (size_t)s->max_lut * 8 + 3 * 256 * 8));
         for (int h = 0; h < 2; ++h) {

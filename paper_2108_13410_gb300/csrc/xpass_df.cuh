@@ -19,8 +19,9 @@
 // Layout in HBM while a call runs ("blocked double-float"): every block of 16 amplitudes
 // (256 bytes of complex128) holds the 16 high (re, im) float pairs, then the 16 low pairs.
 // The first pass of a call splits the complex128 amplitudes of its tiles as it reads them and
-// the last one writes them back as complex128 (conversion kernels of their own took 2.1 of the
-// 24.4 ms of a five-step call at 27 qubits).  The high (low) halves of a tile form an ordinary
+// the last one writes them back as complex128 (against conversion kernels of their own, 27 qubits:
+// one step 9.53 -> 8.51 ms, five 24.1 -> 23.1, forty 151.9 -> 151.0; the two converting passes are
+// bound by arithmetic and take half of what the kernels' two passes over the state took).  The high (low) halves of a tile form an ordinary
 // complex64-like tile under a tensor map with doubled strides (base, base + 128 bytes), so
 // the pass loads a tile pair by two TMA copies and reuses the stage layouts of the
 // complex64 kernel (xpass_tma.cuh).  The pass applies unnormalised Walsh-Hadamard
@@ -75,7 +76,12 @@ __device__ __forceinline__ void df_rotate(u64 (&h)[NR], u64 (&l)[NR], unsigned m
 // (high, low) by TMA into one buffer per CTA (two CTAs per SM); the next pair's load is
 // issued as soon as the current pair's last stage has been read from shared memory, and
 // both halves go back by per-thread stores from registers while that load is in flight.
-template <bool MERGED, bool ROT>
+// RAW, bit 0: the tiles hold complex128 amplitudes (the call's first pass), bit 1: write them back as
+// such (its last).  Only those two passes carry a conversion: as a branch taken at run time it
+// cost every pass registers (spills of 8 to 16 bytes in the merged ones) and long calls more than
+// it saved (32 qubits, 20 steps: 211.4 ms a step with conversion kernels, 215.4 with the branch,
+// 209.9 so).
+template <bool MERGED, bool ROT, int RAW>
 __global__ void __launch_bounds__(NT, 2) k_xpass_df(float2 *__restrict__ state, const double *__restrict__ recs,
                                                     const double *__restrict__ recs2,
                                                     int rec_stride, int tiles_shift, int *__restrict__ err_flag,
@@ -203,7 +209,7 @@ __global__ void __launch_bounds__(NT, 2) k_xpass_df(float2 *__restrict__ state, 
         u64 *tl = reinterpret_cast<u64 *>(buf + (1 << LT));
         u64 h[NR], l[NR];
         // ---- stage A: registers = local 8..11 ----
-        if (P.raw & 1) {
+        if constexpr ((RAW & 1) != 0) {
             // complex128 amplitudes under the two maps: a block's first eight in the high tile's
             // row, the others in the low tile's; all are read before a half is written
             const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(tlo & 8 ? tl : th);
@@ -330,7 +336,7 @@ __global__ void __launch_bounds__(NT, 2) k_xpass_df(float2 *__restrict__ state, 
             // blocked layout: amplitude g = 16 m + j has its high pair at float2 index
             // 32 m + j and its low pair at 32 m + 16 + j
             dst = reinterpret_cast<u64 *>(state) + 2 * (gbase + toff_a) + tlo;
-            if (P.raw & 2) {
+            if constexpr ((RAW & 2) != 0) {
                 double2 *o = reinterpret_cast<double2 *>(state) + gbase + toff_a + tlo;
 #pragma unroll
                 for (int r = 0; r < NR; ++r) o[P.roff_a[r]] = df_join(h[r], l[r]);
@@ -341,7 +347,7 @@ __global__ void __launch_bounds__(NT, 2) k_xpass_df(float2 *__restrict__ state, 
         } else {
             df_renorm(h, l);
             dst = reinterpret_cast<u64 *>(state) + 2 * (gbase + toff_c) + tlo;
-            if (P.raw & 2) {
+            if constexpr ((RAW & 2) != 0) {
                 double2 *o = reinterpret_cast<double2 *>(state) + gbase + toff_c + tlo;
 #pragma unroll
                 for (int r = 0; r < NR; ++r) o[P.roff_c[r]] = df_join(h[r], l[r]);

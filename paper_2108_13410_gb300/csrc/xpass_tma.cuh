@@ -59,8 +59,6 @@ struct TmaPass {
                                 // with a Z layer C is in the scaled table)
     int adj_u[3][2];            // adjoint, tangent form: X qubits of the factor group per
                                 // class not yet un-rotated when stage s reads its terms
-    int raw;                    // double-float passes: bit 0 the tiles hold complex128 amplitudes
-                                // (first pass of a call), bit 1 write them back as such (last)
     int adj_u2[3][2];           // the same for the second round of a shared reverse pass
                                 // (the previous factor group; stages run C, B, A)
 };
