@@ -2,35 +2,18 @@
 // terms and the density of states (sm_103a).
 //
 // All of them read the state and are bound by that where the arithmetic allows: GB300 retires
-// about two FP64 operations per clock and SM, so complex64 sums run in FP32 (products over
-// 16 amplitudes, then an error-free two-float accumulator per thread, converted to FP64 once
-// per block), the parity words of an amplitude are a tile word, a thread word and a register
-// word (no table look-up per amplitude), and of an X string only one amplitude of every pair
-// is visited.  Blocks write partial sums; k_finish adds them in a fixed order.
+// about two FP64 operations per clock and SM, so complex64 products are summed in FP32 over runs
+// of eight amplitudes and a thread's runs in FP64 (sums that never leave FP32, as two floats, run
+// 0 to 15% faster, but overflow where these do not), the parity words of an amplitude are a tile
+// word, a thread word and a register word (no table look-up per amplitude), and of an X string
+// only one amplitude of every pair is visited.  Blocks write partial sums; k_finish adds them in a
+// fixed order.
 // A tile is 4096 consecutive amplitudes (registers bits 8..11, threads bits 0..7) or, for the
 // X terms of the energy, one tile of an X pass (kernels.cuh).
 #pragma once
 #include "kernels.cuh"
 
 namespace qsim {
-
-// Per-thread accumulator: FP64, or for complex64 an unevaluated sum of two floats (Knuth's
-// two-sum keeps every rounding error, so it is as exact as FP64 partial sums of floats).
-template <typename R> struct Acc;
-template <> struct Acc<double> {
-    double h = 0.0;
-    __device__ __forceinline__ void add(double x) { h += x; }
-    __device__ __forceinline__ double value() const { return h; }
-};
-template <> struct Acc<float> {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
-        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
-        h = s;
-    }
-    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
-};
 
 // n - 2 k without a conversion instruction (quarter rate); k < 2^22.  FP64 sums take it from a
 // table in shared memory: the FP64 pipe is what bounds them.
@@ -51,6 +34,36 @@ __device__ __forceinline__ float flip_sign(float x, unsigned odd) {
 __device__ __forceinline__ double flip_sign(double x, unsigned odd) {
     return __longlong_as_double(__double_as_longlong(x) ^ ((long long)odd << 63));
 }
+
+// g += s; l += the rounding error of it (complex64)
+__device__ __forceinline__ void add_keep(float &g, float &l, float s) {
+    const float h = __fadd_rn(g, s), b = __fsub_rn(h, g);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(g, __fsub_rn(h, b)), __fsub_rn(s, b)));
+    g = h;
+}
+__device__ __forceinline__ void add_keep(double &g, double &, double s) { g += s; }
+
+// A thread's FP64 sum over the runs of its tiles.  complex64: two runs of eight at a time, of whose
+// sum the rounding error is kept, so that one FP64 addition takes sixteen amplitudes (halves:
+// the sum of two finite runs may be beyond FP32); complex128: one run of sixteen.
+template <typename R> struct Runs;
+template <> struct Runs<double> {
+    double h;
+    static __device__ __forceinline__ constexpr int run(int) { return 0; }
+    __device__ __forceinline__ void add(double a, double) { h += a; }
+    __device__ __forceinline__ double value() const { return h; }
+};
+template <> struct Runs<float> {
+    double h;
+    float l;
+    static __device__ __forceinline__ constexpr int run(int r) { return r / RED_RUN; }
+    __device__ __forceinline__ void add(float a, float b) {
+        float g = 0.5f * a;
+        add_keep(g, l, 0.5f * b);
+        h += (double)g;
+    }
+    __device__ __forceinline__ double value() const { return 2.0 * (h + (double)l); }
+};
 
 // Parity words of 4096-amplitude tiles: tile word from byte tables over bits 12.., thread word
 // over bits 0..7, register columns over bits 8..11.
@@ -96,8 +109,8 @@ __device__ __forceinline__ void diag_terms(R p, uint32_t a, uint32_t b, const R 
 }
 
 // partial sums [norm, sum_i p_i (nA - 2 oddA(i)), sum_i p_i (nB - 2 oddB(i)), <Z_zmask>], p = |psi|^2
-// (the middle two only if SUMS, the last only if Z).  27 qubits in complex64: 0.15 ms, 0.21 with
-// the sums (0.16 at the measured copy rate); 0.66 ms with four table look-ups per amplitude and
+// (the middle two only if SUMS, the last only if Z).  27 qubits in complex64: 0.15 ms, 0.18 with
+// the sums (0.16 at the measured copy rate; 0.30 with an FP64 addition per run); 0.66 ms with four table look-ups per amplitude and
 // an FP64 add per eight amplitudes and value.  24 qubits in complex128 (FP64-bound): 0.10 ms
 // for the norm, 0.31 before.
 template <typename R, bool SUMS, bool Z>
@@ -118,7 +131,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_diag(const typename C2<R
     const int t = threadIdx.x;
     const long long dim = 1ll << n, ntiles = n > LT ? dim >> LT : 1;
     const unsigned zt = __popc(t & (unsigned)zmask & 255u);
-    Acc<R> acc[4];
+    Runs<R> acc[4] = {};
     for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const V *p0 = psi + (tile << LT) + t;
         V v[NR];
@@ -128,9 +141,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_diag(const typename C2<R
         uint32_t ta = 0, tb = 0;
         if (SUMS) { tile_word(tab, tile, ta, tb); ta ^= q.ta; tb ^= q.tb; }
         const unsigned zz = zt + __popcll(((unsigned long long)tile << LT) & zmask);
-        R f[4] = {0, 0, 0, 0};
+        R f[2][4] = {};
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
+            const int k8 = Runs<R>::run(r);
             const R p = fma(v[r].y, v[r].y, v[r].x * v[r].x);
             uint32_t a = ta, b = tb;
             if (SUMS) {
@@ -138,12 +152,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_diag(const typename C2<R
                 for (int k = 0; k < RB; ++k)
                     if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
             }
-            diag_terms<R, SUMS>(p, a, b, wt, (R)nA, (R)nB, f);
-            if (Z) f[3] += flip_sign(p, (zz + __popc((unsigned)(zmask >> TB) & (unsigned)r)) & 1u);
+            diag_terms<R, SUMS>(p, a, b, wt, (R)nA, (R)nB, f[k8]);
+            if (Z) f[k8][3] += flip_sign(p, (zz + __popc((unsigned)(zmask >> TB) & (unsigned)r)) & 1u);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (k == 0 || (SUMS && k < 3) || (Z && k == 3)) acc[k].add(f[k]);
+            if (k == 0 || (SUMS && k < 3) || (Z && k == 3)) acc[k].add(f[0][k], f[1][k]);
     }
     double out[4];
 #pragma unroll
@@ -162,7 +176,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_xpair(const typename C2<
     psi += (long long)blockIdx.y * state_stride;
     const long long pairs = 1ll << (n - 1), low = (1ll << top) - 1;
     const long long stride = (long long)gridDim.x * RED_THREADS;
-    Acc<R> acc;
+    double acc = 0.0;
     for (long long j0 = blockIdx.x * (long long)RED_THREADS + threadIdx.x; j0 < pairs; j0 += stride * RED_RUN) {
         V x[RED_RUN], y[RED_RUN];
 #pragma unroll
@@ -175,9 +189,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_xpair(const typename C2<
         R f = 0;
 #pragma unroll
         for (int u = 0; u < RED_RUN; ++u) f = fma(x[u].y, y[u].y, fma(x[u].x, y[u].x, f));
-        acc.add(f);
+        acc += (double)f;
     }
-    double out[2] = {2.0 * acc.value(), 0.0};
+    double out[2] = {2.0 * acc, 0.0};
     block_store<2>(out, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
 }
 
@@ -191,7 +205,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_dot(const typename C2<R>
     b += (long long)blockIdx.y * state_stride;
     const long long dim = 1ll << n;
     const long long stride = (long long)gridDim.x * RED_THREADS;
-    Acc<R> re, im;
+    double out[2] = {0.0, 0.0};
     for (long long i0 = blockIdx.x * (long long)RED_THREADS + threadIdx.x; i0 < dim; i0 += stride * RED_RUN) {
         V x[RED_RUN], y[RED_RUN];
 #pragma unroll
@@ -206,10 +220,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_dot(const typename C2<R>
             f0 = fma(x[u].y, y[u].y, fma(x[u].x, y[u].x, f0));
             f1 = fma(-x[u].y, y[u].x, fma(x[u].x, y[u].y, f1));
         }
-        re.add(f0);
-        im.add(f1);
+        out[0] += (double)f0;
+        out[1] += (double)f1;
     }
-    double out[2] = {re.value(), im.value()};
     block_store<2>(out, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
 }
 
@@ -219,8 +232,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_dot(const typename C2<R>
 // registers, through shared memory in the three stage layouts; the first pass also the
 // diagonal sums), then the X strings that no tile holds (stars of the unitary gauge; below 12
 // qubits all X terms, and the diagonal ones in a role of their own).  One read per pass plus
-// half a read per string.  27 qubits in complex64: 0.59 ms (three reads, 0.48 at the copy rate),
-// 1.5 with a diagonal pass of its own; 24 qubits with twelve stars in complex128: 1.6 ms (41 FP64
+// half a read per string.  27 qubits in complex64: 0.68 ms (three reads, 0.48 at the copy rate; 0.58
+// with sums of two floats; half as many FP64 additions, as in k_reduce_diag, cost registers: 0.70),
+// 1.5 with a diagonal pass of its own; 24 qubits with twelve stars in complex128: 1.8 ms (41 FP64
 // operations per amplitude), 4.2 with a reduction per star; 18 qubits with nine stars 25 us in
 // two launches, 150 in 24.
 // ---------------------------------------------------------------------------
@@ -248,6 +262,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
     __shared__ uint2 tab[3 * 256];
     __shared__ double sh[NT / 32][EN_NV];
     __shared__ R wt[2][33];
+    constexpr int RUN = sizeof(R) == 4 ? RED_RUN : NR;
     V *tile_s = reinterpret_cast<V *>(smem_raw);
     const int t = threadIdx.x;
     const int roles = P.np * P.gp;
@@ -261,7 +276,26 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
         load_weights<R>(wt, P.nA, P.nB);
     }
     __syncthreads();
-    Acc<R> acc[5];
+    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    // norm and diagonal sums of a tile's amplitudes
+    auto diag_sums = [&](const V (&v)[NR], long long tau) {
+        uint32_t ta, tb;
+        tile_word(tab, tau, ta, tb);
+        ta ^= q.ta; tb ^= q.tb;
+#pragma unroll
+        for (int r0 = 0; r0 < NR; r0 += RUN) {
+            R f[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int r = r0; r < r0 + RUN; ++r) {
+                uint32_t a = ta, b = tb;
+#pragma unroll
+                for (int k = 0; k < RB; ++k)
+                    if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
+                diag_terms<R, true>(fma(v[r].y, v[r].y, v[r].x * v[r].x), a, b, wt, (R)P.nA, (R)P.nB, f);
+            }
+            acc[0] += (double)f[0]; acc[1] += (double)f[1]; acc[2] += (double)f[2];
+        }
+    };
     if (role < P.np) {
         const int c = P.c[role], next = P.next[role];
         auto g = [&](int j) { return j < c ? j : next + (j - c); };   // global bit of tile bit j
@@ -286,6 +320,9 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
                 v[r] = p[off];
             }
         };
+        // eight pairs of every register bit; the bits' sums add up with their rounding errors
+        // kept in l0, l1 (complex64: two-sum)
+        R l0 = 0, l1 = 0;
         auto pairs = [&](const V (&v)[NR], unsigned mask, unsigned cl, R &g0, R &g1) {
 #pragma unroll
             for (int k = 0; k < RB; ++k) {
@@ -294,7 +331,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
 #pragma unroll
                 for (int r = 0; r < NR; ++r)
                     if (!((r >> k) & 1)) s = fma(v[r].y, v[r | (1 << k)].y, fma(v[r].x, v[r | (1 << k)].x, s));
-                if ((cl >> k) & 1u) g1 += s; else g0 += s;
+                if ((cl >> k) & 1u) add_keep(g1, l1, s); else add_keep(g0, l0, s);
             }
         };
         const int tlo = t & 15, thi = t >> 4;
@@ -309,21 +346,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
                 load(v, tau);
             }
             R g0 = 0, g1 = 0;
-            if (role == 0) {
-                uint32_t ta, tb;
-                tile_word(tab, tau, ta, tb);
-                ta ^= q.ta; tb ^= q.tb;
-                R f[4] = {0, 0, 0, 0};
-#pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    uint32_t a = ta, b = tb;
-#pragma unroll
-                    for (int k = 0; k < RB; ++k)
-                        if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
-                    diag_terms<R, true>(fma(v[r].y, v[r].y, v[r].x * v[r].x), a, b, wt, (R)P.nA, (R)P.nB, f);
-                }
-                acc[0].add(f[0]); acc[1].add(f[1]); acc[2].add(f[2]);
-            }
+            if (role == 0) diag_sums(v, tau);
             pairs(v, rot >> 8, cls >> 8, g0, g1);
 #pragma unroll
             for (int r = 0; r < NR; ++r) tile_s[swz(t | (r << TB))] = v[r];
@@ -340,10 +363,12 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
                 for (int r = 0; r < NR; ++r) v[r] = tile_s[swz(tlo | (r << 4) | (thi << 8))];
                 pairs(v, rot >> 4, cls >> 4, g0, g1);
             }
-            acc[3].add((R)2 * g0);
-            acc[4].add((R)2 * g1);
+            acc[3] += (double)g0;
+            acc[4] += (double)g1;
             __syncthreads();
         }
+        acc[3] += (double)l0;
+        acc[4] += (double)l1;
     } else {
         const int b0 = (int)blockIdx.x - roles;
         for (long long tau = b0; tau < ntiles; tau += P.gm) {
@@ -352,41 +377,32 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
 #pragma unroll
             for (int r = 0; r < NR; ++r)
                 v[r] = i0 + (r << TB) < dim ? psi[i0 + (r << TB)] : mk<R>((R)0, (R)0);
-            if (diag) {
-                uint32_t ta, tb;
-                tile_word(tab, tau, ta, tb);
-                ta ^= q.ta; tb ^= q.tb;
-                R f[4] = {0, 0, 0, 0};
-#pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    uint32_t a = ta, b = tb;
-#pragma unroll
-                    for (int k = 0; k < RB; ++k)
-                        if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
-                    diag_terms<R, true>(fma(v[r].y, v[r].y, v[r].x * v[r].x), a, b, wt, (R)P.nA, (R)P.nB, f);
-                }
-                acc[0].add(f[0]); acc[1].add(f[1]); acc[2].add(f[2]);
-            }
+            if (diag) diag_sums(v, tau);
             for (int j = 0; j < P.nmasks; ++j) {
                 const long long m = (long long)P.mask[j];
                 const long long top = 1ll << (63 - __clzll(m));
-                R s = 0;
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    const long long i = i0 + (r << TB);
-                    if (i < dim && !(i & top)) {
-                        const V y = psi[i ^ m];
-                        s = fma(v[r].y, y.y, fma(v[r].x, y.x, s));
+                for (int r0 = 0; r0 < NR; r0 += RUN) {
+                    R s = 0;
+#pragma unroll
+                    for (int r = r0; r < r0 + RUN; ++r) {
+                        const long long i = i0 + (r << TB);
+                        if (i < dim && !(i & top)) {
+                            const V y = psi[i ^ m];
+                            s = fma(v[r].y, y.y, fma(v[r].x, y.x, s));
+                        }
                     }
+                    if ((P.mask_cls >> j) & 1) acc[4] += (double)s; else acc[3] += (double)s;
                 }
-                if ((P.mask_cls >> j) & 1) acc[4].add((R)2 * s); else acc[3].add((R)2 * s);
             }
         }
     }
+    acc[3] *= 2.0;                 // every pair was visited once
+    acc[4] *= 2.0;
     const int w = t >> 5;
 #pragma unroll
     for (int k = 0; k < EN_NV; ++k) {
-        const double x = k < 5 ? warp_sum(acc[k].value()) : 0.0;
+        const double x = k < 5 ? warp_sum(acc[k < 5 ? k : 0]) : 0.0;
         if ((t & 31) == 0) sh[w][k] = x;
     }
     __syncthreads();
