@@ -444,46 +444,57 @@ __global__ void __launch_bounds__(RED_THREADS) k_finish(const double *__restrict
 // ---------------------------------------------------------------------------
 // Density of states of Z~ = -sum_l sigma^z_l (Sec. V): weight of the amplitudes with k links
 // in sigma^z = -1.  Each thread keeps its own column of bins in shared memory (no atomics) and
-// adds one sum per number of links set among its register bits; complex64 weights are exact
-// products in two-float sums on the FP32 pipes.  partials[(b * gridDim.x + blk) * nbins + k].
-// 27 qubits in complex64 0.40 ms (one FP64 shared-memory atomic per amplitude: 12.5), 24 qubits
-// in complex128 0.09 (1.4).
+// adds one sum per number of links set among its register bits, products and sums in FP64 (bins
+// differ by orders of magnitude).  partials[(b * gridDim.x + blk) * nbins + k].  What bounds it
+// is the FP64 pipe: 2.3 operations an amplitude; the conversion instruction, of the same rate,
+// is replaced by integer operations for floats that are normal or zero.  27 qubits in complex64
+// 0.56 ms (1.15 with the instruction, 0.41 with product pairs in two floats, whose bins were up
+// to 28 times further off; one FP64 shared-memory atomic per amplitude: 12.5), 24 qubits in
+// complex128 0.09 (1.4).
 // ---------------------------------------------------------------------------
-template <typename R> struct Bin;
-template <> struct Bin<double> {
-    typedef double T;
-    static __device__ __forceinline__ T zero() { return 0.0; }
-    static __device__ __forceinline__ void weigh(T &s, double2 a) { s = fma(a.y, a.y, fma(a.x, a.x, s)); }
-    static __device__ __forceinline__ T sum(T a, T b) { return a + b; }
-    static __device__ __forceinline__ double value(T a) { return a; }
-};
-template <> struct Bin<float> {
-    typedef float2 T;      // high, low
-    static __device__ __forceinline__ T zero() { return make_float2(0.f, 0.f); }
-    static __device__ __forceinline__ void add(T &s, float x, float e) {
-        const float h = __fadd_rn(s.x, x), b = __fsub_rn(h, s.x);
-        s.y = __fadd_rn(s.y, __fadd_rn(e, __fadd_rn(__fsub_rn(s.x, __fsub_rn(h, b)), __fsub_rn(x, b))));
-        s.x = h;
+// |x| of a float that is normal or zero as a double, by integer operations (the conversion
+// instruction runs at the FP64 rate), and whether it is such a float
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x) & 0x7fffffffu;
+    return __hiloint2double((int)(u ? (u >> 3) + 0x38000000u : 0u), (int)(u << 29));
+}
+__device__ __forceinline__ bool widens(float x) {
+    const unsigned u = __float_as_uint(x) & 0x7fffffffu;
+    return u == 0u || u - 0x00800000u < 0x7f000000u;
+}
+__device__ __forceinline__ bool widens(float2 a) { return widens(a.x) && widens(a.y); }
+__device__ __forceinline__ bool widens(double2) { return true; }
+template <bool FAST> __device__ __forceinline__ double2 as_double(float2 a) {
+    return FAST ? make_double2(widen(a.x), widen(a.y)) : make_double2((double)a.x, (double)a.y);
+}
+template <bool FAST> __device__ __forceinline__ double2 as_double(double2 a) { return a; }
+
+// a thread's 16 amplitudes into its column of bins
+template <bool FAST, bool FOLD, typename V>
+__device__ __forceinline__ void dos_tile(const V (&v)[NR], double *col, unsigned reg) {
+    double s[RB + 1] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const double2 a = as_double<FAST>(v[r]);
+        double *bin = &col[__popc((unsigned)r & reg) * RED_THREADS];
+        double &sum = FOLD ? s[(r & 1) + ((r >> 1) & 1) + ((r >> 2) & 1) + (r >> 3)] : *bin;
+        sum = fma(a.y, a.y, fma(a.x, a.x, sum));
     }
-    static __device__ __forceinline__ void weigh(T &s, float2 a) {
-        const float p = __fmul_rn(a.x, a.x), q = __fmul_rn(a.y, a.y);
-        add(s, p, __fmaf_rn(a.x, a.x, -p));
-        add(s, q, __fmaf_rn(a.y, a.y, -q));
+    if (FOLD) {
+#pragma unroll
+        for (int k = 0; k <= RB; ++k) col[k * RED_THREADS] += s[k];
     }
-    static __device__ __forceinline__ T sum(T a, T b) { add(a, b.x, b.y); return a; }
-    static __device__ __forceinline__ double value(T a) { return (double)a.x + (double)a.y; }
-};
+}
 
 template <typename R>
 __global__ void __launch_bounds__(RED_THREADS) k_dos(const typename C2<R>::T *__restrict__ psi, int n,
                                                     long long state_stride, unsigned long long linkmask, int nbins,
                                                     double *__restrict__ partials) {
     using V = typename C2<R>::T;
-    typedef Bin<R> B;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    typename B::T *bins = reinterpret_cast<typename B::T *>(smem_raw);     // [nbins][RED_THREADS]
+    double *bins = reinterpret_cast<double *>(smem_raw);                   // [nbins][RED_THREADS]
     const int t = threadIdx.x;
-    for (int k = 0; k < nbins; ++k) bins[k * RED_THREADS + t] = B::zero();
+    for (int k = 0; k < nbins; ++k) bins[k * RED_THREADS + t] = 0.0;
     psi += (long long)blockIdx.y * state_stride;
     const long long dim = 1ll << n, ntiles = n > LT ? dim >> LT : 1;
     const unsigned reg = (unsigned)(linkmask >> TB) & 15u;                 // links among the register bits
@@ -494,35 +505,17 @@ __global__ void __launch_bounds__(RED_THREADS) k_dos(const typename C2<R>::T *__
 #pragma unroll
         for (int r = 0; r < NR; ++r)
             v[r] = n >= LT || (r << TB) + t < dim ? p0[r << TB] : mk<R>((R)0, (R)0);
-        typename B::T *col = bins + (kt + __popcll(((unsigned long long)tile << LT) & linkmask)) * RED_THREADS + t;
-        if (reg == 15u || reg == 0u) {
-            typename B::T s[RB + 1];
+        double *col = bins + (kt + __popcll(((unsigned long long)tile << LT) & linkmask)) * RED_THREADS + t;
+        bool fast = true;
 #pragma unroll
-            for (int k = 0; k <= RB; ++k) s[k] = B::zero();
-            if (reg) {
-#pragma unroll
-                for (int r = 0; r < NR; ++r) B::weigh(s[(r & 1) + ((r >> 1) & 1) + ((r >> 2) & 1) + (r >> 3)], v[r]);
-#pragma unroll
-                for (int k = 0; k <= RB; ++k) col[k * RED_THREADS] = B::sum(col[k * RED_THREADS], s[k]);
-            } else {
-#pragma unroll
-                for (int r = 0; r < NR; ++r) B::weigh(s[0], v[r]);
-                col[0] = B::sum(col[0], s[0]);
-            }
-        } else {
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                typename B::T s = B::zero();
-                B::weigh(s, v[r]);
-                typename B::T *c = col + __popc((unsigned)r & reg) * RED_THREADS;
-                *c = B::sum(*c, s);
-            }
-        }
+        for (int r = 0; r < NR; ++r) fast = fast && widens(v[r]);
+        if (reg == 15u) { if (fast) dos_tile<true, true>(v, col, reg); else dos_tile<false, true>(v, col, reg); }
+        else { if (fast) dos_tile<true, false>(v, col, reg); else dos_tile<false, false>(v, col, reg); }
     }
     __syncthreads();
     for (int k = t >> 5; k < nbins; k += RED_THREADS / 32) {
         double s = 0.0;
-        for (int j = t & 31; j < RED_THREADS; j += 32) s += B::value(bins[k * RED_THREADS + j]);
+        for (int j = t & 31; j < RED_THREADS; j += 32) s += bins[k * RED_THREADS + j];
         s = warp_sum(s);
         if ((t & 31) == 0) partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * nbins + k] = s;
     }
