@@ -276,6 +276,9 @@ qs_status qs_dos(qs_sim *sim, double *out);
  * buffers, and the register-staged kernel; complex128: the register-staged kernel) on
  * the bound state, which is overwritten, and keeps the fastest (QS_OPT_XPASS,
  * QS_OPT_TMA_BUFFERS, QS_OPT_TMA_STORE, QS_OPT_SHARED_BUFFERS, QS_OPT_SHARED_KERNEL).
+ * Where the default configuration has kernels of its own (QS_OPT_XPASS 0: small states in
+ * one launch; QS_OPT_PLAN: larger tiles) it is timed too, and small states with at least
+ * the 11 steps from which long calls take that form.
  * Outputs the choice and its ms per step (host). */
 qs_status qs_autotune(qs_sim *sim, int n_steps, int *best_xpass, int *best_buffers, int *best_store,
                       int *best_shared_buffers, int *best_shared_kernel, double *best_ms_per_step);
