@@ -94,7 +94,8 @@ typedef enum {
                                  register-staged kernel, 2 the persistent TMA kernel
                                  (complex64; complex128: the double-float passes)    */
     QS_OPT_TMA_BUFFERS = 5,   /* shared-memory tile buffers per CTA of the TMA kernel:
-                                 2 (three CTAs per SM) or 3 (default; two CTAs per SM) */
+                                 2 (three CTAs per SM; keeps the tiles of 12 qubits,
+                                 QS_OPT_PLAN) or 3 (default; two CTAs per SM)         */
     QS_OPT_ADJOINT = 6,       /* complex64 adjoint reverse pass: bit 0 set = register-
                                  staged kernel, clear = TMA kernel (default).  TMA
                                  kernel, 0 (default): one psi/lambda tile-pair buffer

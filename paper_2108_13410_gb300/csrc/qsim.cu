@@ -1230,10 +1230,11 @@ bool default_plan(const qs_sim *s, const std::vector<int> &k) {
     return true;
 }
 
-// 2^13 tiles: by default (no kernel, plan or buffer option set) where they save passes.
+// 2^13 tiles: by default (no kernel chosen, plan, buffers and stores at their defaults) where they
+// save passes.
 bool wide_schedule(const qs_sim *s) {
     return !s->wide_maps.empty() && s->xpass_impl == 0 && s->plan_code == 0 && !s->shared_kernel_set &&
-           s->shared_kernel == 1 && s->nbuf_shared == 0 && s->tma_store;
+           s->shared_kernel == 1 && s->nbuf == 3 && s->nbuf_shared == 0 && s->tma_store;
 }
 
 // Unitary gauge with shared passes: the X layer of factor group k is H^n D_X H^n
