@@ -5,7 +5,6 @@
 // sequencing on the bound stream, and FP64 reductions read back to the host.
 #include <cuda_runtime.h>
 
-#include <atomic>
 #include <cmath>
 #include <functional>
 #include <cstdio>
@@ -1733,19 +1732,45 @@ ScanParams scan12_params(const qs_sim *s, int n_points, int n_steps, int order, 
     return P;
 }
 
-// Shared-memory limits that no lattice changes, once per device.
-void set_fixed_attributes(int dev) {
-    static std::atomic<unsigned long long> done{0};
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (done.load() & bit) return;
-    const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaFuncSetAttribute(k_energy<double>, A, (1 << LT) * 16);
-    cudaFuncSetAttribute(k_dos<float>, A, 64 * RED_THREADS * 8);
-    cudaFuncSetAttribute(k_dos<double>, A, 64 * RED_THREADS * 8);
-    cudaFuncSetAttribute(k_xpass_wide<W_GROUPS, 16>, A, 226 * 1024);
-    cudaFuncSetAttribute(k_xpass_wide<W_SLICE4, W_SLICE_WARPS>, A, 226 * 1024);
-    cudaFuncSetAttribute(k_xpass_wide<W_SLICE3, W_SLICE_WARPS>, A, 226 * 1024);
-    done.fetch_or(bit);
+// Shared-memory limits of the kernels on the current device, for the largest phase table that
+// qs_create allows: a limit that followed each new simulator's table made launches of larger
+// ones fail.  The kernel that is set last tells whether they are set.
+void set_kernel_limits() {
+    const int lut = 33 * 33, tabs = lut * 8 + 3 * 256 * 8 + 1024;
+    const int last = (1 << LT) * 16 + lut * 16;
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, k_xpass<float>) == cudaSuccess && at.maxDynamicSharedSizeBytes == last) return;
+    auto limit = [](auto kern, int bytes) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    limit(k_energy<double>, (1 << LT) * 16);
+    limit(k_dos<float>, 64 * RED_THREADS * 8);
+    limit(k_dos<double>, 64 * RED_THREADS * 8);
+    limit(k_xpass_wide<W_GROUPS, 16>, 226 * 1024);
+    limit(k_xpass_wide<W_SLICE4, W_SLICE_WARPS>, 226 * 1024);
+    limit(k_xpass_wide<W_SLICE3, W_SLICE_WARPS>, 226 * 1024);
+    for (int nb = 2; nb <= 3; ++nb)
+        for (int v = 0; v < 8; ++v) limit(xpass_tma_kernel(nb, v & 1, (v >> 1) & 1, (v >> 2) & 1), nb * TMA_TILE_BYTES + tabs);
+    for (int v = 0; v < 16; ++v)
+        limit(df_kernel(v & 1, (v >> 1) & 1, v >> 2), 2 * TMA_TILE_BYTES + lut * 32 + 3 * 256 * 8 + 1024);
+    limit(k_adj_wl<3, 12, 1, 0>, 6 * TMA_TILE_BYTES + tabs);
+    for (int h = 0; h < 2; ++h) {
+        limit(h ? k_xpass_wl<2, 8, 3, true> : k_xpass_wl<2, 8, 3, false>, 2 * TMA_TILE_BYTES + tabs);
+        limit(h ? k_xpass_wl<3, 8, 2, true> : k_xpass_wl<3, 8, 2, false>, 3 * TMA_TILE_BYTES + tabs);
+        limit(h ? k_xpass_wl<6, 24, 1, true> : k_xpass_wl<6, 24, 1, false>, 6 * TMA_TILE_BYTES + tabs);
+    }
+    for (int v = 0; v < 3; ++v) {
+        const bool tn = v >= 1, mg = v == 2;
+        limit(adj_tma_kernel(2, tn, mg), 4 * TMA_TILE_BYTES + tabs);
+        for (int ea = 0; ea < 2; ++ea) limit(adj_tma_kernel(1, tn, mg, ea != 0), 2 * TMA_TILE_BYTES + tabs);
+    }
+    const int adj64 = 2 * (1 << LT) * 16 + lut * 16;
+    limit(k_adj_xpass<float>, adj64);
+    limit(k_adj_xpass<double>, adj64);
+    limit(k_apply_h_pass<float>, adj64);
+    limit(k_apply_h_pass<double>, adj64);
+    limit(k_xpass<double>, last);
+    limit(k_xpass<float>, last);
 }
 
 qs_status check_ready(qs_sim *s) {
@@ -1846,42 +1871,8 @@ qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, dev);
         if (s->sm_count < 1) s->sm_count = 1;
-        set_fixed_attributes(dev);
-        for (int nb = 2; nb <= 3; ++nb)
-            for (int v = 0; v < 8; ++v)
-                cudaFuncSetAttribute(xpass_tma_kernel(nb, v & 1, (v >> 1) & 1, (v >> 2) & 1),
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tma_smem_bytes(s, nb, true));
-        for (int v = 0; v < 16; ++v)
-            cudaFuncSetAttribute(df_kernel(v & 1, (v >> 1) & 1, v >> 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)df_smem_bytes(s));
-        cudaFuncSetAttribute(k_adj_wl<3, 12, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(2 * (size_t)TMA_TILE_BYTES * 3 + 1024 + (size_t)s->max_lut * 8 + 3 * 256 * 8));
-        for (int h = 0; h < 2; ++h) {
-            cudaFuncSetAttribute(h ? k_xpass_wl<2, 8, 3, true> : k_xpass_wl<2, 8, 3, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tma_smem_bytes(s, 2, true));
-            cudaFuncSetAttribute(h ? k_xpass_wl<3, 8, 2, true> : k_xpass_wl<3, 8, 2, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tma_smem_bytes(s, 3, true));
-            cudaFuncSetAttribute(h ? k_xpass_wl<6, 24, 1, true> : k_xpass_wl<6, 24, 1, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tma_smem_bytes(s, 6, true));
-        }
-        int adj64 = (int)(2 * (1 << LT) * 16 + (size_t)(s->nA + 1) * (s->nB + 1) * 16);
-        cudaFuncSetAttribute(k_adj_xpass<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
-        cudaFuncSetAttribute(k_adj_xpass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
-        cudaFuncSetAttribute(k_apply_h_pass<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
-        cudaFuncSetAttribute(k_apply_h_pass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, adj64);
-        for (int v = 0; v < 3; ++v) {
-            const bool tn = v >= 1, mg = v == 2;
-            cudaFuncSetAttribute(adj_tma_kernel(2, tn, mg), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(4 * TMA_TILE_BYTES + 1024 + (size_t)s->max_lut * 8 + 3 * 256 * 8));
-            for (int ea = 0; ea < 2; ++ea)
-                cudaFuncSetAttribute(adj_tma_kernel(1, tn, mg, ea != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(2 * TMA_TILE_BYTES + 1024 + (size_t)s->max_lut * 8 + 3 * 256 * 8));
-        }
-
+        set_kernel_limits();
     }
-    size_t smem64 = (size_t)(1 << LT) * 16 + (size_t)s->max_lut * 16;
-    cudaFuncSetAttribute(k_xpass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64);
-    cudaFuncSetAttribute(k_xpass<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64);
     *out = s;
     return QS_OK;
 }
