@@ -320,8 +320,10 @@ int qs_plan(const qs_sim *sim, int *qubits_per_pass, int max);
 
 /* Failure-detection self-test: launches a kernel that waits on an mbarrier which
  * never completes, with the same bounded wait as the TMA X pass, limited to
- * limit_ms (0 < limit_ms <= 2000).  Expected result: QS_ERR_TIMEOUT, with the
- * context still usable afterwards. */
+ * limit_ms (0 < limit_ms <= 2000), and for a bound state that would run on the chip
+ * with an exchange (QS_OPT_XPASS) one CTA of such a run, which waits for the others'
+ * amplitudes under the same limit.  Expected result: QS_ERR_TIMEOUT (flag 2, with the
+ * second wait 3), with the context still usable afterwards and the state as it was. */
 qs_status qs_selftest_wait(qs_sim *sim, double limit_ms);
 
 /* Checkpoint: write (qs_save) or read (qs_load) the bound state with a header

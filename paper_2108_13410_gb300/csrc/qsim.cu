@@ -2641,6 +2641,22 @@ qs_status qs_selftest_wait(qs_sim *s, double limit_ms) {
     long long cycles = (long long)(limit_ms * (double)khz);
     k_wait_probe<<<1, 32, 0, s->stream>>>(s->d_err, cycles);
     CKL(s); s->launches++;
+    if (s->state[0] && s->passes.size() <= 2 && resident_fits(s) && s->res.two) {
+        // one CTA of a resident run: its poll for the amplitudes of the others runs out, and it
+        // leaves before it stores any
+        qs_status st;
+        const size_t bytes = 2 * (size_t)s->batch * (size_t)s->res.rec_bytes;
+        if ((st = resident_mail(s)) != QS_OK) return st;
+        if ((st = grow(s, &s->d_rec, &s->d_rec_cap, (bytes + 7) / 8, false)) != QS_OK) return st;
+        CK(s, cudaMemsetAsync(s->d_rec, 0, bytes, s->stream));
+        ResParams P = s->res;
+        P.nops = 2;
+        P.last_z = 1;
+        P.wait = cycles;
+        s->res_mail_ready = false;
+        CK(s, resident_launch(P, s->state[0], s->d_rec, s->d_res_mail, s->d_err, s->stream, 1));
+        s->launches++;
+    }
     CK(s, cudaStreamSynchronize(s->stream));
     return check_device_flag(s);
 }

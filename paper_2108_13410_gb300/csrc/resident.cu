@@ -584,7 +584,7 @@ __global__ void __launch_bounds__((1 << (M - R)) + 32, min_ctas(M, R, sizeof(typ
                 for (int r = 0; r < NRG; ++r)
                     if (!arrived(x[r])) { all = false; x[r] = recv(p + off_of(set, r)); }
                 if (all) break;
-                if (clock64() - t0 > 2000000000ll) {      // about a second
+                if (clock64() - t0 > P.wait) {
                     atomicOr(err_flag, 1);
                     s_ok = 0;
                     break;
@@ -795,6 +795,7 @@ bool resident_plan(ResParams &P, int arith, int n, int batch, int sm_count) {
     const long long room = (long long)per_sm * sm_count / P.tiles;
     if (room < 1) return false;
     P.batch = batch;
+    P.wait = 2000000000ll;      // about a second
     P.groups = (int)(room < batch ? room : batch);
     if (P.groups > RES_MAX_GROUPS) P.groups = RES_MAX_GROUPS;
     return true;
@@ -831,12 +832,12 @@ cudaError_t resident_tables(const ResParams &P, const RecGeom &G, const double *
 }
 
 cudaError_t resident_launch(const ResParams &P, void *state, const void *recs, void *mail, int *err_flag,
-                            cudaStream_t stream) {
+                            cudaStream_t stream, int ctas) {
     int threads = 0;
     size_t smem = 0;
     const ResKernel k = kernel_of(P, &threads, &smem, P.tab_bytes);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(P.tiles * P.groups));
+    cfg.gridDim = dim3((unsigned)(ctas ? ctas : P.tiles * P.groups));
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = P.smem;
     cfg.stream = stream;

@@ -27,6 +27,7 @@ struct ResParams {
     uint32_t colA[RES_MAXQ], colB[RES_MAXQ];   // Z-layer terms containing each qubit
     uint32_t xcolA[RES_MAXQ], xcolB[RES_MAXQ]; // Hadamard-basis X terms containing each qubit
     uint32_t cls;              // bit q: qubit q is a vertex (tau^x)
+    long long wait;            // limit of a poll, SM cycles
 };
 
 // Fills arith, n, M, c, two, tiles, groups and the sizes; false if the state does not fit the chip
@@ -39,8 +40,9 @@ cudaError_t resident_mail_clear(const ResParams &P, void *mail, cudaStream_t str
 // Records of factor groups op0 .. op0 + nops - 1 (rec_bytes each, group-major).
 cudaError_t resident_tables(const ResParams &P, const RecGeom &G, const double *in, size_t ncpl, const RecInline &X,
                             bool inl, int op0, int nops, void *recs, int sm_count, cudaStream_t stream);
+// (ctas: that many of the run's CTAs only, whose polls for the others' amplitudes run out)
 cudaError_t resident_launch(const ResParams &P, void *state, const void *recs, void *mail, int *err_flag,
-                            cudaStream_t stream);
+                            cudaStream_t stream, int ctas = 0);
 constexpr int RES_MAX_GROUPS = 4096;
 
 }  // namespace qsim

@@ -64,10 +64,36 @@ def test_one_to_three_groups(form, Lx, Ly, periodic, dtype, steps, order):
 
 
 @gpu
+@pytest.mark.parametrize("form,Lx,Ly", [("gh", 3, 2), ("ug", 3, 3), ("ug", 4, 2)])
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+def test_a_poll_that_runs_out(form, Lx, Ly, dtype):
+    """One CTA of a run alone: it gives up (bit 1 of the flag), leaves the state as it was and its
+    tile in a mail box, which the next run clears."""
+    import torch
+    from paper_2108_13410_gb300 import Simulator
+    from paper_2108_13410_gb300.qsim import QsError, qs_selftest_wait
+    lat = OracleLattice(Lx, Ly, True, form)
+    sim = Simulator(Lx, Ly, form=form, dtype=dtype)
+    psi0 = synth.random_state(lat.n_qubits, seed=5)
+    s = O.schedule_linear(0.6, 12)
+    ref = O.evolve(lat, Couplings(0.4, 0.7), s, 0.05, 2, psi0=psi0)
+    host = torch.from_numpy(psi0.reshape(1, -1)).to(sim.state.dtype)
+    for _ in range(2):
+        sim.upload(host)
+        with pytest.raises(QsError) as e:
+            qs_selftest_wait(sim.h, 5.0)
+        assert e.value.status == 5 and "flag 3" in str(e.value)
+        assert torch.equal(sim.download(), host)
+        sim.launch_count()
+        sim.evolve([(0.4, 0.7)], s, 0.05, 2)
+        assert np.linalg.norm(sim.download()[0].numpy() - ref) <= (1e-5 if dtype == "c64" else 1e-10)
+        assert sim.launch_count() == 2
+
+
+@gpu
 @pytest.mark.parametrize("form,Lx,Ly", [("gh", 3, 2), ("ug", 3, 3)])
 def test_boxes_are_cleared_after_a_wait_that_ran_out(form, Lx, Ly):
-    """A timeout (here of the self test's own wait) leaves the boxes in doubt: the next run clears
-    them."""
+    """A timeout leaves the boxes in doubt: the next run clears them."""
     import torch
     from paper_2108_13410_gb300 import Simulator
     from paper_2108_13410_gb300.qsim import QsError, qs_selftest_wait
