@@ -577,13 +577,13 @@ def ug32_leg(local, dev, stream):
                     "xpass": kern, "step_hbm_gbs": npass * alg / (ms / 1000.0) / 1e9,
                     "norm_minus_1": float(sim.expect(QS_NORM)[0] - 1.0)}
         if key == "c128":
-            # the in-place split into the blocked double-float layout and the join back run
-            # once per call, inside the time above: the call time minus the X-pass
-            # launches' own event times is the split, the join and the launch gaps
+            # the first pass splits complex128 into the double-float layout and the last one
+            # joins it, inside their own times: the call time minus the X-pass launches'
+            # event times is the operator records and the launch gaps
             xpass_ms = kinds[0][0] + kinds[1][0]
             out[key]["arithmetic"] = "double-float (two floats per real number, FP32 pipes)"
             out[key]["xpass_ms_per_step"] = xpass_ms / n
-            out[key]["split_join_and_gaps_ms_per_call"] = ms - xpass_ms
+            out[key]["records_and_gaps_ms_per_call"] = ms - xpass_ms
         elif key == "c128_fp64":
             out[key]["arithmetic"] = "FP64"
         del sim

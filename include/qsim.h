@@ -87,8 +87,10 @@ typedef enum {
                                  the bound stream (read with qs_profile_read)        */
     QS_OPT_GRAPH = 3,         /* 1: qs_evolve replays its launches as a CUDA graph    */
     QS_OPT_XPASS = 4,         /* X-pass kernel: 0 auto: small states (up to 2^19
-                                 amplitudes in all; any number of states of up to 12
-                                 qubits) run in one launch with the state on the chip
+                                 amplitudes in all; any number of states of up to 11
+                                 qubits, in complex64 12; complex128 beyond 12 qubits
+                                 more than four states 2^18 amplitudes)
+                                 run in one launch with the state on the chip
                                  (beyond 12 qubits calls of up to 3 or at least 12
                                  factor groups), others as 2; 1 the
                                  register-staged kernel, 2 the persistent TMA kernel
@@ -138,7 +140,8 @@ typedef enum {
                                  for states of fewer than 13 qubits.  With the default
                                  plan, complex64 unitary-gauge runs of one state may use
                                  larger tiles (13 qubits, then up to 10 per pass) where
-                                 they save passes: 21 to 23 and 29 to 33 qubits.       */
+                                 they save passes: 22 and 30 to 32 qubits; qs_plan then
+                                 still names the plan of the 2^12 tiles.               */
     QS_OPT_SCAN_BUFFERS = 12, /* qs_scan_mixed: 32 KB tile buffers per CTA of the
                                  larger lattice's passes, 2 or 3 (two CTAs per SM) or 4
                                  or 6 (one CTA per SM; a pass keeps buffers - 1 loads in
@@ -313,8 +316,8 @@ qs_status qs_scan_mixed(qs_sim *sim12, const qs_couplings *p12, int n12, qs_sim 
 qs_status qs_autotune_plan(qs_sim *sim, int n_steps, int *qubits_per_pass, int max, int *n_passes,
                            double *best_ms_per_step);
 
-/* The current pass plan: qubits fused by each tiled X pass (the first 12), host output of
- * at most max entries; returns the number of passes (0 for states smaller than one tile,
+/* The current pass plan: qubits fused by each tiled X pass over tiles of 12 qubits (the
+ * first 12; larger tiles, QS_OPT_PLAN, are not shown), host output of at most max entries; returns the number of passes (0 for states smaller than one tile,
  * -1 on a bad argument). */
 int qs_plan(const qs_sim *sim, int *qubits_per_pass, int max);
 

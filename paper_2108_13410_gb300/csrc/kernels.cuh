@@ -57,7 +57,7 @@ struct PassDesc {
 //   phase pairs (u, s) of exp(i phi(nA_odd, nB_odd))], where exp(i t) = (1 - u) + i s,
 //   u = 1 - cos t, s = sin t (u keeps full relative precision for small angles);
 //   then the Hadamard-basis X table (unitary gauge) and, at tan_off, the tangent form
-//   (t_sigma, t_tau, C, 0) of the X layer (dev_tan_triple) followed by the Z table
+//   (t_sigma, t_tau, C, 0) of the X layer (dev_tan) followed by the Z table
 //   scaled by C (dev_scaled_pair; same layout as the plain Z table).
 __host__ __device__ inline int record_doubles(int nA, int nB) {
     int r = 4 + 2 * (nA + 1) * (nB + 1);

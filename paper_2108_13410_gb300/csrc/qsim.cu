@@ -340,7 +340,7 @@ void build_tma_passes(qs_sim *s) {
 
 // Passes over 2^13 tiles: 13 qubits, then windows of 9 or 10 qubits above a chunk of 4 or 3 (a
 // window of 9 may start on qubits that are already done).  Only where they are fewer than the
-// passes of 2^12 tiles: 21 to 23 and 29 to 33 qubits.  4x4 torus (32 qubits, 32 GiB): 4 passes
+// passes of 2^12 tiles (of the lattices there are: 22 and 30 to 32 qubits).  4x4 torus (32 qubits, 32 GiB): 4 passes
 // per step instead of 6.
 void build_wide_passes(qs_sim *s) {
     s->wide.clear();
@@ -1300,8 +1300,9 @@ bool df_schedule(const qs_sim *s) {
 // over passes per step: complex64 2^19 amplitudes 0.66 (19 qubits), 0.59 (4 x 17), 0.77 (64 x
 // 13), 2^20 1.12 (20 qubits), 1.15 (4 x 18), 1.64 (16 x 16); double-float 2^18 0.48 (18 qubits),
 // 0.72 (4 x 16), 2^19 0.69 (19 qubits), 0.75 (4 x 17) but 1.4 (64 x 13), 2^20 1.24 (4 x 18);
-// FP64 2^18 0.37 to 0.51 (64 x 12).
-
+// FP64 2^18 0.37 to 0.51 (64 x 12), 2^19 0.58 (gauge-Higgs) and 0.98 (unitary gauge), beyond
+// 0.58 to 0.68 and 0.89 to 1.03 (152 to 8192 x 12): the limit is where the unitary gauge stops
+// gaining, the gauge-Higgs form would gain beyond it.
 bool resident_size(const qs_sim *s) {
     if (s->n < LT || (s->n == LT && s->dtype == QS_C64)) return true;
     const long long amps = (long long)s->batch << s->n;
@@ -1350,8 +1351,12 @@ qs_status resident_mail(qs_sim *s) {
 
 // A call runs resident by default (QS_OPT_XPASS auto, shared passes on, the default pass
 // plan, no per-pass profiling).  Beyond one tile, runs of 4 to 11 factor groups keep one
-// launch per pass, whose number qs_launch_count reports to callers that rely on it; a single
-// step of 18 qubits (two groups, five launches there) takes 42 us in a loop, resident 26.
+// launch per pass, and that is not for speed: tests pin the launches of 18-qubit complex64 calls
+// of 11 groups, and the rule makes no difference between sizes, forms and precisions.  Measured,
+// resident / passes, us a call in a loop: 18 qubits, 2 groups 26 / 42; 4 groups 43 / 65 (unitary
+// gauge), 36 / 48 (gauge-Higgs), complex128 89 / 134, 70 / 102; 11 groups 93 / 149, 71 / 102,
+// 207 / 373, 150 / 251; 13 qubits, gauge-Higgs, 4 groups 31 / 44, 58 / 93; 16, 17 and 19 qubits
+// likewise (0.55 to 0.78).
 bool resident_groups(const qs_sim *s, size_t groups) { return s->n <= LT || groups <= 3 || groups >= 12; }
 
 bool resident_call(qs_sim *s, size_t nops, int steps_per_renorm_unit) {

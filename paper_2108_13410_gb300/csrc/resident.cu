@@ -175,9 +175,10 @@ struct AF64 {
     template <int N> static __device__ __forceinline__ void tidy(V (&)[N]) {}
 };
 
-// Exchange words: a word that holds EMPTY has not arrived yet.  EMPTY is a signalling NaN in
-// either half (and as a double), which no arithmetic result is; everything that is sent
-// comes out of a butterfly or a product.
+// Exchange words: a word that holds EMPTY has not arrived yet.  EMPTY is a signalling NaN as a
+// double and in its low half as a float (its high half is a quiet one), which no arithmetic
+// result is; everything that is sent comes out of a butterfly or a product, and the whole word is
+// compared.
 constexpr u64 EMPTY = 0x7ff4dead7fa0deadull;
 
 __device__ __forceinline__ bool arrived(u64 w) { return w != EMPTY; }
@@ -382,8 +383,11 @@ constexpr int min_ctas(int M, int R, bool df, bool two) {
 }
 
 // Threads 2^(M - R), then one helper warp that loads the table and the tangents of the next
-// pass and takes the fence between clearing and sending (1000 cycles) off the workers' path;
-// blockIdx.x = group * tiles + tile of the state.  Named barriers: 1 the workers, 2 a pass has
+// pass and takes the fence between clearing and sending (1000 cycles) off the workers' path: that
+// relies on a fence covering what its thread has observed through a CTA barrier (cumulativity, as
+// in a grid barrier, where one thread's fence stands for its block) and on no store of the CTA
+// overtaking the barrier behind the fence; the memory model's own release pattern would have every
+// sending thread fence.  blockIdx.x = group * tiles + tile of the state.  Named barriers: 1 the workers, 2 a pass has
 // received and cleared (workers arrive, helper waits), 3 the next table is there and the
 // clears are ordered (helper arrives, workers wait).
 template <class A, int M, int R, bool HAD, bool TWO>

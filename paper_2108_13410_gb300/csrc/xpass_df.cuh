@@ -20,10 +20,10 @@
 // (256 bytes of complex128) holds the 16 high (re, im) float pairs, then the 16 low pairs.
 // The first pass of a call splits the complex128 amplitudes of its tiles as it reads them and
 // the last one writes them back as complex128 (against conversion kernels of their own, 27 qubits:
-// one step 9.53 -> 8.51 ms, five 24.1 -> 23.1, forty 151.9 -> 151.0; the two converting passes are
-// bound by arithmetic and take half of what the kernels' two passes over the state took).  The high (low) halves of a tile form an ordinary
-// complex64-like tile under a tensor map with doubled strides (base, base + 128 bytes), so
-// the pass loads a tile pair by two TMA copies and reuses the stage layouts of the
+// one step 9.53 -> 8.51 ms, five 24.1 -> 23.1, forty 151.9 -> 151.0; what the two converting
+// passes take more is about half of what the kernels took).  The high (low) halves of a tile form
+// an ordinary complex64-like tile under a tensor map with doubled strides (base, base + 128
+// bytes), so the pass loads a tile pair by two TMA copies and reuses the stage layouts of the
 // complex64 kernel (xpass_tma.cuh).  The pass applies unnormalised Walsh-Hadamard
 // butterflies on the pass's qubits (the unitary-gauge X layer H^n D_X H^n and the Z layer
 // between transforms, Sec. II), optionally the diagonal table with its scale, and (MERGED)

@@ -5,7 +5,7 @@
 // tile: H on the pass's qubits, optionally a diagonal table (the Hadamard-basis X layer D_X with
 // its 2^-n, or the Z layer) and H again.  The passes are bound by HBM, so what counts is how many
 // a step takes: tiles of 2^12 amplitudes (12 qubits, then 8 per pass) need four passes to visit
-// 29 to 32 qubits and three for 21 to 23, tiles of 2^13 with rows of 64 bytes (13 qubits, then
+// 30 to 32 qubits and three for 22 (the sizes that lattices have there), tiles of 2^13 with rows of 64 bytes (13 qubits, then
 // up to 10 per pass) three and two, i.e. 4 instead of 6 and 2 instead of 4 passes per step
 // (32 qubits: 73 -> 56 ms a step, 30 qubits 18.0 -> 12.7).  Rows of 64 bytes, which only a window
 // of ten qubits needs, cost 8% of the rate (plain pass 12.7 instead of 11.8 ms).
