@@ -2,12 +2,11 @@
 // terms and the density of states (sm_103a).
 //
 // All of them read the state and are bound by that where the arithmetic allows: GB300 retires
-// about two FP64 operations per clock and SM, so complex64 products are summed in FP32 over runs
-// of eight amplitudes and a thread's runs in FP64 (sums that never leave FP32, as two floats, run
-// 0 to 15% faster, but overflow where these do not), the parity words of an amplitude are a tile
-// word, a thread word and a register word (no table look-up per amplitude), and of an X string
-// only one amplitude of every pair is visited.  Blocks write partial sums; k_finish adds them in a
-// fixed order.
+// about two FP64 operations per clock and SM, so complex64 sums run in FP32 without rounding
+// error, products and sums as pairs of floats, and go to FP64 once per sixteen amplitudes.  The
+// parity words of an amplitude are a tile word, a thread word and a register word (no table
+// look-up per amplitude), and of an X string only one amplitude of every pair is visited.  Blocks
+// write partial sums; k_finish adds them in a fixed order.
 // A tile is 4096 consecutive amplitudes (registers bits 8..11, threads bits 0..7) or, for the
 // X terms of the energy, one tile of an X pass (kernels.cuh).
 #pragma once
@@ -43,26 +42,61 @@ __device__ __forceinline__ void add_keep(float &g, float &l, float s) {
 }
 __device__ __forceinline__ void add_keep(double &g, double &, double s) { g += s; }
 
-// A thread's FP64 sum over the runs of its tiles.  complex64: two runs of eight at a time, of whose
-// sum the rounding error is kept, so that one FP64 addition takes sixteen amplitudes (halves:
-// the sum of two finite runs may be beyond FP32); complex128: one run of sixteen.
+// A product of two amplitudes' parts, Re(conj(a) b).  complex64: without rounding error, as a sum of
+// two floats: observables are small differences of sums of order one.  (With rounded products in
+// runs of eight they were up to ten times further off than with one amplitude of a small state
+// per FP64 addition: 18 qubits, norm 1.1e-9 against 5.1e-10, X strings 2.7e-9 against 5.4e-10; so
+// 6e-16 and 1e-16.)
+__device__ __forceinline__ double product(double2 a, double2 b) { return fma(a.y, b.y, a.x * b.x); }
+__device__ __forceinline__ float2 product(float2 a, float2 b) {
+    float h = __fmul_rn(a.x, b.x), l = __fmaf_rn(a.x, b.x, -h);
+    const float q = __fmul_rn(a.y, b.y);
+    l = __fadd_rn(l, __fmaf_rn(a.y, b.y, -q));
+    add_keep(h, l, q);
+    return make_float2(h, l);
+}
+
+// A thread's sum of products, in FP64 over runs.  complex64: two runs of eight at a time, so that
+// one FP64 addition takes sixteen amplitudes (halves: the sum of two finite runs may be beyond
+// FP32); l takes the parts that do not fit the runs.  complex128: one run of sixteen.
 template <typename R> struct Runs;
 template <> struct Runs<double> {
+    typedef double T;
     double h;
     static __device__ __forceinline__ constexpr int run(int) { return 0; }
+    // f += p, f += w p, f += Re(conj(a) b)
+    __device__ __forceinline__ void term(double &f, double p) { f += p; }
+    __device__ __forceinline__ void term(double &f, double p, double w) { f = fma(p, w, f); }
+    __device__ __forceinline__ void pair(double &f, double2 a, double2 b) { f = fma(a.y, b.y, fma(a.x, b.x, f)); }
+    static __device__ __forceinline__ double flip(double p, unsigned odd) { return flip_sign(p, odd); }
     __device__ __forceinline__ void add(double a, double) { h += a; }
     __device__ __forceinline__ double value() const { return h; }
 };
 template <> struct Runs<float> {
+    typedef float2 T;
     double h;
     float l;
     static __device__ __forceinline__ constexpr int run(int r) { return r / RED_RUN; }
-    __device__ __forceinline__ void add(float a, float b) {
-        float g = 0.5f * a;
-        add_keep(g, l, 0.5f * b);
-        h += (double)g;
+    __device__ __forceinline__ void term(float &f, float2 p) {
+        add_keep(f, l, p.x);
+        l = __fadd_rn(l, p.y);
     }
-    __device__ __forceinline__ double value() const { return 2.0 * (h + (double)l); }
+    __device__ __forceinline__ void term(float &f, float2 p, float w) {
+        const float q = __fmul_rn(p.x, w);
+        add_keep(f, l, q);
+        l = __fadd_rn(l, __fmaf_rn(p.y, w, __fmaf_rn(p.x, w, -q)));
+    }
+    __device__ __forceinline__ void pair(float &f, float2 a, float2 b) { term(f, product(a, b)); }
+    static __device__ __forceinline__ float2 flip(float2 p, unsigned odd) {
+        return make_float2(flip_sign(p.x, odd), flip_sign(p.y, odd));
+    }
+    __device__ __forceinline__ void add(float a, float b) {
+        float g = 0.5f * a, e = 0.f;
+        add_keep(g, e, 0.5f * b);
+        h += (double)g;
+        l = __fmaf_rn(2.0f, e, l);
+    }
+    __device__ __forceinline__ double value() const { return 2.0 * h + (double)l; }
 };
 
 // Parity words of 4096-amplitude tiles: tile word from byte tables over bits 12.., thread word
@@ -97,22 +131,12 @@ __device__ __forceinline__ void tile_word(const uint2 *tab, long long tile, uint
     b = x.y ^ y.y ^ z.y;
 }
 
-// |psi|^2 sums of one amplitude set: f[0] norm, and if SUMS f[1], f[2] weighted by nA - 2 oddA,
-// nB - 2 oddB
-template <typename R, bool SUMS>
-__device__ __forceinline__ void diag_terms(R p, uint32_t a, uint32_t b, const R (*w)[33], R nA, R nB, R (&f)[4]) {
-    f[0] += p;
-    if (SUMS) {
-        f[1] = fma(p, weight(w[0], nA, __popc(a)), f[1]);
-        f[2] = fma(p, weight(w[1], nB, __popc(b)), f[2]);
-    }
-}
-
 // partial sums [norm, sum_i p_i (nA - 2 oddA(i)), sum_i p_i (nB - 2 oddB(i)), <Z_zmask>], p = |psi|^2
-// (the middle two only if SUMS, the last only if Z).  27 qubits in complex64: 0.15 ms, 0.18 with
-// the sums (0.16 at the measured copy rate; 0.30 with an FP64 addition per run); 0.66 ms with four table look-ups per amplitude and
-// an FP64 add per eight amplitudes and value.  24 qubits in complex128 (FP64-bound): 0.10 ms
-// for the norm, 0.31 before.
+// (the middle two only if SUMS, the last only if Z).  27 qubits in complex64: 0.17 ms, 0.22 with
+// a Z string, 0.36 with the sums (0.16 at the measured copy rate; 0.15, 0.16 and 0.18 with rounded
+// products in runs of eight); 0.66 ms with four table look-ups per amplitude and an FP64 add
+// per eight amplitudes and value.  24 qubits in complex128 (FP64-bound): 0.10 ms for the norm,
+// 0.31 before.
 template <typename R, bool SUMS, bool Z>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_diag(const typename C2<R>::T *__restrict__ psi, int n,
                                                             long long state_stride, const uint32_t *__restrict__ colA,
@@ -145,15 +169,17 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_diag(const typename C2<R
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const int k8 = Runs<R>::run(r);
-            const R p = fma(v[r].y, v[r].y, v[r].x * v[r].x);
-            uint32_t a = ta, b = tb;
+            const typename Runs<R>::T p = product(v[r], v[r]);
+            acc[0].term(f[k8][0], p);
             if (SUMS) {
+                uint32_t a = ta, b = tb;
 #pragma unroll
                 for (int k = 0; k < RB; ++k)
                     if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
+                acc[1].term(f[k8][1], p, weight(wt[0], (R)nA, __popc(a)));
+                acc[2].term(f[k8][2], p, weight(wt[1], (R)nB, __popc(b)));
             }
-            diag_terms<R, SUMS>(p, a, b, wt, (R)nA, (R)nB, f[k8]);
-            if (Z) f[k8][3] += flip_sign(p, (zz + __popc((unsigned)(zmask >> TB) & (unsigned)r)) & 1u);
+            if (Z) acc[3].term(f[k8][3], Runs<R>::flip(p, (zz + __popc((unsigned)(zmask >> TB) & (unsigned)r)) & 1u));
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -176,7 +202,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_xpair(const typename C2<
     psi += (long long)blockIdx.y * state_stride;
     const long long pairs = 1ll << (n - 1), low = (1ll << top) - 1;
     const long long stride = (long long)gridDim.x * RED_THREADS;
-    double acc = 0.0;
+    Runs<R> acc = {};
     for (long long j0 = blockIdx.x * (long long)RED_THREADS + threadIdx.x; j0 < pairs; j0 += stride * RED_RUN) {
         V x[RED_RUN], y[RED_RUN];
 #pragma unroll
@@ -188,10 +214,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_xpair(const typename C2<
         }
         R f = 0;
 #pragma unroll
-        for (int u = 0; u < RED_RUN; ++u) f = fma(x[u].y, y[u].y, fma(x[u].x, y[u].x, f));
-        acc += (double)f;
+        for (int u = 0; u < RED_RUN; ++u) acc.pair(f, x[u], y[u]);
+        acc.add(f, (R)0);
     }
-    double out[2] = {2.0 * acc, 0.0};
+    double out[2] = {2.0 * acc.value(), 0.0};
     block_store<2>(out, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
 }
 
@@ -205,7 +231,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_dot(const typename C2<R>
     b += (long long)blockIdx.y * state_stride;
     const long long dim = 1ll << n;
     const long long stride = (long long)gridDim.x * RED_THREADS;
-    double out[2] = {0.0, 0.0};
+    Runs<R> re = {}, im = {};
     for (long long i0 = blockIdx.x * (long long)RED_THREADS + threadIdx.x; i0 < dim; i0 += stride * RED_RUN) {
         V x[RED_RUN], y[RED_RUN];
 #pragma unroll
@@ -217,12 +243,13 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_dot(const typename C2<R>
         R f0 = 0, f1 = 0;
 #pragma unroll
         for (int u = 0; u < RED_RUN; ++u) {
-            f0 = fma(x[u].y, y[u].y, fma(x[u].x, y[u].x, f0));
-            f1 = fma(-x[u].y, y[u].x, fma(x[u].x, y[u].y, f1));
+            re.pair(f0, x[u], y[u]);
+            im.pair(f1, mk<R>(x[u].x, -x[u].y), mk<R>(y[u].y, y[u].x));
         }
-        out[0] += (double)f0;
-        out[1] += (double)f1;
+        re.add(f0, (R)0);
+        im.add(f1, (R)0);
     }
+    double out[2] = {re.value(), im.value()};
     block_store<2>(out, partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * RED_NV);
 }
 
@@ -232,11 +259,11 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_dot(const typename C2<R>
 // registers, through shared memory in the three stage layouts; the first pass also the
 // diagonal sums), then the X strings that no tile holds (stars of the unitary gauge; below 12
 // qubits all X terms, and the diagonal ones in a role of their own).  One read per pass plus
-// half a read per string.  27 qubits in complex64: 0.68 ms (three reads, 0.48 at the copy rate; 0.58
-// with sums of two floats; half as many FP64 additions, as in k_reduce_diag, cost registers: 0.70),
-// 1.5 with a diagonal pass of its own; 24 qubits with twelve stars in complex128: 1.8 ms (41 FP64
-// operations per amplitude), 4.2 with a reduction per star; 18 qubits with nine stars 25 us in
-// two launches, 150 in 24.
+// half a read per string.  27 qubits in complex64: 0.79 ms (three reads, 0.48 at the copy rate; the
+// exact diagonal sums cost the first pass its registers: 0.68 with rounded products), 1.5 with a
+// diagonal pass of its own; 24 qubits with twelve stars 0.30 ms, in complex128 1.35 (FP64 pipe; 1.8
+// when tiles whose partner visits a string's pairs did not skip it), 4.2 with a reduction per
+// star; 18 qubits with nine stars 25 us in two launches, 150 in 24.
 // ---------------------------------------------------------------------------
 constexpr int EN_NV = 8;
 constexpr int EN_MASKS = 64;
@@ -262,7 +289,6 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
     __shared__ uint2 tab[3 * 256];
     __shared__ double sh[NT / 32][EN_NV];
     __shared__ R wt[2][33];
-    constexpr int RUN = sizeof(R) == 4 ? RED_RUN : NR;
     V *tile_s = reinterpret_cast<V *>(smem_raw);
     const int t = threadIdx.x;
     const int roles = P.np * P.gp;
@@ -276,25 +302,28 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
         load_weights<R>(wt, P.nA, P.nB);
     }
     __syncthreads();
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    Runs<R> acc[3] = {};           // diagonal sums
+    double xs[2] = {0.0, 0.0};     // X terms by class, every pair once
     // norm and diagonal sums of a tile's amplitudes
     auto diag_sums = [&](const V (&v)[NR], long long tau) {
         uint32_t ta, tb;
         tile_word(tab, tau, ta, tb);
         ta ^= q.ta; tb ^= q.tb;
+        R f[2][3] = {};
 #pragma unroll
-        for (int r0 = 0; r0 < NR; r0 += RUN) {
-            R f[4] = {0, 0, 0, 0};
+        for (int r = 0; r < NR; ++r) {
+            const int k8 = Runs<R>::run(r);
+            const typename Runs<R>::T p = product(v[r], v[r]);
+            uint32_t a = ta, b = tb;
 #pragma unroll
-            for (int r = r0; r < r0 + RUN; ++r) {
-                uint32_t a = ta, b = tb;
-#pragma unroll
-                for (int k = 0; k < RB; ++k)
-                    if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
-                diag_terms<R, true>(fma(v[r].y, v[r].y, v[r].x * v[r].x), a, b, wt, (R)P.nA, (R)P.nB, f);
-            }
-            acc[0] += (double)f[0]; acc[1] += (double)f[1]; acc[2] += (double)f[2];
+            for (int k = 0; k < RB; ++k)
+                if ((r >> k) & 1) { a ^= q.ra[k]; b ^= q.rb[k]; }
+            acc[0].term(f[k8][0], p);
+            acc[1].term(f[k8][1], p, weight(wt[0], (R)P.nA, __popc(a)));
+            acc[2].term(f[k8][2], p, weight(wt[1], (R)P.nB, __popc(b)));
         }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) acc[k].add(f[0][k], f[1][k]);
     };
     if (role < P.np) {
         const int c = P.c[role], next = P.next[role];
@@ -363,12 +392,12 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
                 for (int r = 0; r < NR; ++r) v[r] = tile_s[swz(tlo | (r << 4) | (thi << 8))];
                 pairs(v, rot >> 4, cls >> 4, g0, g1);
             }
-            acc[3] += (double)g0;
-            acc[4] += (double)g1;
+            xs[0] += (double)g0;
+            xs[1] += (double)g1;
             __syncthreads();
         }
-        acc[3] += (double)l0;
-        acc[4] += (double)l1;
+        xs[0] += (double)l0;
+        xs[1] += (double)l1;
     } else {
         const int b0 = (int)blockIdx.x - roles;
         for (long long tau = b0; tau < ntiles; tau += P.gm) {
@@ -381,28 +410,30 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
             for (int j = 0; j < P.nmasks; ++j) {
                 const long long m = (long long)P.mask[j];
                 const long long top = 1ll << (63 - __clzll(m));
+                if (tau & (top >> LT)) continue;     // the partner tile visits the pairs
+                R f[2] = {0, 0};
+                Runs<R> sum = {};
 #pragma unroll
-                for (int r0 = 0; r0 < NR; r0 += RUN) {
-                    R s = 0;
+                for (int r0 = 0; r0 < NR; r0 += RED_RUN) {
+                    V y[RED_RUN];
 #pragma unroll
-                    for (int r = r0; r < r0 + RUN; ++r) {
-                        const long long i = i0 + (r << TB);
-                        if (i < dim && !(i & top)) {
-                            const V y = psi[i ^ m];
-                            s = fma(v[r].y, y.y, fma(v[r].x, y.x, s));
-                        }
+                    for (int r = 0; r < RED_RUN; ++r) {
+                        const long long i = i0 + ((r0 + r) << TB);
+                        y[r] = i < dim && !(i & top) ? psi[i ^ m] : mk<R>((R)0, (R)0);
                     }
-                    if ((P.mask_cls >> j) & 1) acc[4] += (double)s; else acc[3] += (double)s;
+#pragma unroll
+                    for (int r = 0; r < RED_RUN; ++r) sum.pair(f[Runs<R>::run(r0)], v[r0 + r], y[r]);
                 }
+                sum.add(f[0], f[1]);
+                if ((P.mask_cls >> j) & 1) xs[1] += sum.value(); else xs[0] += sum.value();
             }
         }
     }
-    acc[3] *= 2.0;                 // every pair was visited once
-    acc[4] *= 2.0;
+    const double out[5] = {acc[0].value(), acc[1].value(), acc[2].value(), 2.0 * xs[0], 2.0 * xs[1]};
     const int w = t >> 5;
 #pragma unroll
     for (int k = 0; k < EN_NV; ++k) {
-        const double x = k < 5 ? warp_sum(acc[k < 5 ? k : 0]) : 0.0;
+        const double x = k < 5 ? warp_sum(out[k < 5 ? k : 0]) : 0.0;
         if ((t & 31) == 0) sh[w][k] = x;
     }
     __syncthreads();
