@@ -170,7 +170,9 @@ typedef enum {
  * needs Lx, Ly >= 1.  batch >= 1 independent states share the lattice; each has
  * its own couplings.  Fails with QS_ERR_ARG if the qubit count exceeds 34.
  * Allocates only small device workspaces (term tables, partial sums; at the first
- * call that runs on the chip, two mail boxes of at most 2^19 amplitudes each). */
+ * call that runs on the chip, two mail boxes of at most 2^19 amplitudes each, which
+ * qs_destroy may keep for the device's next simulator: 32 MiB at most, none once the last
+ * one is gone). */
 qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch,
                     qs_sim **out);
 void qs_destroy(qs_sim *sim);

@@ -7,6 +7,7 @@
 
 #include <cmath>
 #include <functional>
+#include <mutex>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -37,6 +38,54 @@ namespace {
 thread_local std::string g_create_error;
 constexpr int RED_BLOCKS = 152 * 4;  // reduction grid per batch element (fixed: deterministic)
 constexpr int RES_SLOTS = 160;       // reduction result slots per readback
+
+// Mail boxes (resident.cu) of destroyed simulators, for the next ones of the same device: a
+// cudaMalloc of 2 MiB or more takes 80 us, as much as the rest of a small state's first call.  At
+// most 32 MiB are kept, none once the device's last simulator is gone.
+struct MailStore {
+    struct Block { void *p; size_t bytes; int dev; };
+    static constexpr size_t LIMIT = 32u << 20;
+    std::mutex mu;
+    std::vector<Block> kept;
+    std::vector<int> sims;      // simulators per device
+
+    void *take(size_t bytes, int dev) {
+        std::lock_guard<std::mutex> g(mu);
+        for (size_t i = 0; i < kept.size(); ++i)
+            if (kept[i].dev == dev && kept[i].bytes == bytes) {
+                void *p = kept[i].p;
+                kept.erase(kept.begin() + i);
+                return p;
+            }
+        return nullptr;
+    }
+    // p: no work on it is left
+    void give(void *p, size_t bytes, int dev) {
+        std::lock_guard<std::mutex> g(mu);
+        size_t total = bytes;
+        for (const Block &b : kept) total += b.bytes;
+        if (bytes < (1u << 20) || total > LIMIT) cudaFree(p);    // (small ones take 3 us)
+        else kept.push_back({p, bytes, dev});
+    }
+    void enter(int dev) {
+        std::lock_guard<std::mutex> g(mu);
+        if ((int)sims.size() <= dev) sims.resize(dev + 1, 0);
+        ++sims[dev];
+        kept.reserve(LIMIT >> 20);      // give() allocates nothing
+    }
+    void leave(int dev) {
+        std::lock_guard<std::mutex> g(mu);
+        if (--sims[dev]) return;
+        for (size_t i = 0; i < kept.size();)
+            if (kept[i].dev == dev) {
+                cudaFree(kept[i].p);
+                kept.erase(kept.begin() + i);
+            } else {
+                ++i;
+            }
+    }
+};
+MailStore g_mail;
 
 // One Trotter factor group: exp(-i tau H_X) (angles per X class), then optionally
 // exp(-i dt H_Z) (plaquette and second-class Z angles).
@@ -117,6 +166,7 @@ struct qs_sim {
     bool res_active = false;               // this call runs resident
     void *d_res_mail = nullptr;            // its mail boxes (allocated at the first call that needs them)
     bool res_mail_ready = false;           // cleared, and no launch on them has timed out since
+    int dev = -1;                          // device of the workspaces (set once they exist)
     int adj_impl = 0;                      // adjoint reverse pass: 0 auto (TMA), 1 register kernel
     int adj_early = 1;                     // one buffer, tangent form: next load issued before the stores
     int sm_count = 0;
@@ -1339,6 +1389,7 @@ bool resident_fits(qs_sim *s) {
 qs_status resident_mail(qs_sim *s) {
     const size_t bytes = resident_mail_bytes(s->res);
     if (!bytes || s->res_mail_ready) return QS_OK;
+    if (!s->d_res_mail) s->d_res_mail = g_mail.take(bytes, s->dev);
     if (!s->d_res_mail && cudaMalloc(&s->d_res_mail, bytes) != cudaSuccess) {
         cudaGetLastError();
         s->d_res_mail = nullptr;
@@ -1877,6 +1928,12 @@ qs_status qs_create(int Lx, int Ly, int boundary, int form, int dtype, int batch
         cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, dev);
         if (s->sm_count < 1) s->sm_count = 1;
         set_kernel_limits();
+        try {
+            g_mail.enter(dev);
+        } catch (const std::exception &) {
+            return fail("host memory");
+        }
+        s->dev = dev;
     }
     *out = s;
     return QS_OK;
@@ -1891,7 +1948,10 @@ void qs_destroy(qs_sim *s) {
     cudaFree(s->d_rec);
     cudaFree(s->d_partials);
     cudaFree(s->d_res);
-    cudaFree(s->d_res_mail);
+    if (s->d_res_mail) {
+        cudaDeviceSynchronize();      // (a run on a stream that was set before, too)
+        g_mail.give(s->d_res_mail, resident_mail_bytes(s->res), s->dev);
+    }
     cudaFree(s->d_adj_part);
     cudaFree(s->d_grad);
     cudaFree(s->d_hrec);
@@ -1907,6 +1967,7 @@ void qs_destroy(qs_sim *s) {
     if (s->h_res) cudaFreeHost(s->h_res);
     if (s->rec_done) cudaEventDestroy(s->rec_done);
     for (auto e : s->ev_pool) cudaEventDestroy(e);
+    if (s->dev >= 0) g_mail.leave(s->dev);
     delete s;
 }
 
