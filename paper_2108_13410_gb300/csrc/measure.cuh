@@ -264,6 +264,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_dot(const typename C2<R>
 // diagonal pass of its own; 24 qubits with twelve stars 0.30 ms, in complex128 1.35 (FP64 pipe; 1.8
 // when tiles whose partner visits a string's pairs did not skip it), 4.2 with a reduction per
 // star; 18 qubits with nine stars 25 us in two launches, 150 in 24.
+// EXACT (complex64): the pairs of the tiles' qubits without rounding error too, ten times their
+// FP32 operations: for states of up to 20 qubits, where a call is launches and latency (at most
+// 6 us more), and for the mean fields of a scan, which were reductions per qubit.  18 qubits:
+// sigma^x energy 1.3e-8 -> 1e-15 from 64 bits.
 // ---------------------------------------------------------------------------
 constexpr int EN_NV = 8;
 constexpr int EN_MASKS = 64;
@@ -277,7 +281,7 @@ struct EnergyParams {
     unsigned long long mask_cls;   // bit j: string j is of class 1
 };
 
-template <typename R>
+template <typename R, bool EXACT>
 __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typename C2<R>::T *__restrict__ psi,
                                                                     long long state_stride,
                                                                     const uint32_t *__restrict__ colA,
@@ -356,11 +360,20 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_energy(const typ
 #pragma unroll
             for (int k = 0; k < RB; ++k) {
                 if (!((mask >> k) & 1u)) continue;
-                R s = 0;
+                R s = 0, l = 0;
 #pragma unroll
-                for (int r = 0; r < NR; ++r)
-                    if (!((r >> k) & 1)) s = fma(v[r].y, v[r | (1 << k)].y, fma(v[r].x, v[r | (1 << k)].x, s));
+                for (int r = 0; r < NR; ++r) {
+                    if ((r >> k) & 1) continue;
+                    if constexpr (EXACT) {
+                        const float2 p = product(v[r], v[r | (1 << k)]);
+                        add_keep(s, l, p.x);
+                        l += p.y;
+                    } else {
+                        s = fma(v[r].y, v[r | (1 << k)].y, fma(v[r].x, v[r | (1 << k)].x, s));
+                    }
+                }
                 if ((cl >> k) & 1u) add_keep(g1, l1, s); else add_keep(g0, l0, s);
+                if (EXACT) { if ((cl >> k) & 1u) l1 += l; else l0 += l; }
             }
         };
         const int tlo = t & 15, thi = t >> 4;

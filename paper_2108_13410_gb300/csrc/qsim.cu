@@ -1799,7 +1799,7 @@ void set_kernel_limits() {
     auto limit = [](auto kern, int bytes) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-    limit(k_energy<double>, (1 << LT) * 16);
+    limit(k_energy<double, false>, (1 << LT) * 16);
     limit(k_dos<float>, 64 * RED_THREADS * 8);
     limit(k_dos<double>, 64 * RED_THREADS * 8);
     limit(k_xpass_wide<W_GROUPS, 16>, 226 * 1024);
@@ -2148,7 +2148,7 @@ qs_status qs_evolve(qs_sim *s, const qs_couplings *c, const double *sv, double d
 // Every term of <H>: per state EN_NV values [norm, sum Z_A, sum Z_B, sum X class 0, class 1] at
 // h_res[b * EN_NV] (one launch and the sum over its blocks; synchronises).
 template <typename R>
-static qs_status energy_terms(qs_sim *s) {
+static qs_status energy_terms(qs_sim *s, bool fields = false) {
     qs_status st;
     const int B = s->batch;
     EnergyParams P;
@@ -2180,7 +2180,8 @@ static qs_status energy_terms(qs_sim *s) {
     P.gm = P.nmasks ? (int)std::min<long long>(ntiles, (long long)s->sm_count * 4) : 0;
     const size_t nblk = (size_t)np * P.gp + P.gm;
     if ((st = grow(s, &s->d_adj_part, &s->adj_part_cap, nblk * B * EN_NV, false)) != QS_OK) return st;
-    k_energy<R><<<dim3((unsigned)nblk, B), NT, np ? (size_t)(1 << LT) * sizeof(V<R>) : 0, s->stream>>>(
+    const auto kern = sizeof(R) == 4 && (fields || s->n <= 20) ? k_energy<R, sizeof(R) == 4> : k_energy<R, false>;
+    kern<<<dim3((unsigned)nblk, B), NT, np ? (size_t)(1 << LT) * sizeof(V<R>) : 0, s->stream>>>(
         (const V<R> *)s->state[0], s->dim, s->d_colA, s->d_colB, P, s->d_adj_part);
     CKL(s); s->launches++;
     k_finish<EN_NV><<<B, RED_THREADS, 0, s->stream>>>(s->d_adj_part, (int)nblk, EN_NV, s->d_res);
@@ -2397,7 +2398,7 @@ qs_status qs_scan(qs_sim *s, const qs_couplings *points, int n_points, const dou
             for (int b = 0; b < cnt; ++b) out[(size_t)(p0 + b) * SCAN_NOBS + k] = v[b];
         };
         // energy, mean plaquette, norm and the mean fields from the terms of one measurement
-        if ((st = s->dtype == QS_C64 ? energy_terms<float>(s) : energy_terms<double>(s)) != QS_OK) return st;
+        if ((st = s->dtype == QS_C64 ? energy_terms<float>(s, true) : energy_terms<double>(s)) != QS_OK) return st;
         const int nl = s->lat.n_links, nv = s->n - s->lat.n_links;
         for (int b = 0; b < cnt; ++b) {
             const Coef q = coefficients(chunk[b], 1.0);

@@ -3,7 +3,8 @@
 Products of floats and the sums of a thread's sixteen amplitudes are kept in two floats, sums beyond
 that in FP64: at most 2^-48 per amplitude and thread, of which a thread takes fewer than 2^10 here,
 so 2^-38 = 3.7e-12 of the sum of the terms' magnitudes (1 for a string, the number of terms for
-their sum).  The single-qubit X terms of an energy are chains of FP32 products and not in here."""
+their sum).  The single-qubit X terms of an energy beyond 20 qubits are chains of FP32 products
+and not in here."""
 import numpy as np
 import pytest
 
@@ -47,6 +48,11 @@ def test_sums_hold_more_than_single_precision(form, Lx, Ly, periodic, kind):
     assert abs(sim.expect(QS_PLAQUETTE, -1)[0] - zsum(plaq) / len(plaq)) <= TOL
     assert abs(sim.energy([(0.0, 0.0, 0.0, 1.0)])[0] + zsum(plaq)) <= len(plaq) * TOL
     assert abs(sim.energy([(0.0, 1.0, 0.0, 0.0)])[0] + zsum(second)) <= len(second) * TOL
+    xs = [q for q, kind in lat.x_single() if kind == "s"]
+    assert abs(sim.energy([(1.0, 0.0, 0.0, 0.0)])[0] + sum(xval(1 << q) for q in xs)) <= len(xs) * TOL
+    if form == "gh":
+        xt = [q for q, kind in lat.x_single() if kind == "t"]
+        assert abs(sim.energy([(0.0, 0.0, 1.0, 0.0)])[0] + sum(xval(1 << q) for q in xt)) <= len(xt) * TOL
     if form == "ug":
         stars = [int(m) for m in lat.x_strings()]
         assert abs(sim.energy([(0.0, 0.0, 1.0, 0.0)])[0] + sum(xval(m) for m in stars)) <= len(stars) * TOL
